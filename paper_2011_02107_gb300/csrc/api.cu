@@ -123,6 +123,13 @@ struct dacp_ctx {
     int emax_rule = 0;                  // E_max bound: 0 Ritz value + residual norm, 1 Ritz-residual rule
     double* mom_d = nullptr;
     int64_t mom_cap = 0;
+    // fixed-point evolution (resident.cu): workspace, grown to the largest launch so far
+    double* fx_emax_d = nullptr;        // [R]
+    int *fx_list_d = nullptr, *fx_status_d = nullptr;   // [R]
+    unsigned* fx_bar_d = nullptr;       // [R]
+    float4* fx_pro_d = nullptr;
+    longlong2* fx_part_d = nullptr;
+    size_t fx_ctas = 0, fx_parts = 0;
 
     // parameters
     std::vector<double> emax, a;
@@ -515,6 +522,120 @@ dacp_status apply_params(dacp_ctx* c) {
     return DACP_OK;
 }
 
+dacp_status set_evolution_coef(dacp_ctx* c, const std::vector<double>& emax);
+
+// Whether the evolution of blocks of b columns runs in fixed point with resident vectors, and how:
+// float64 vectors without pair couplings whose realizations fit a group's shared memory.
+bool fx_usable(const dacp_ctx* c, int b, FxPlan* plan) {
+    if (c->prec != kPrecF64 || c->has_pairs || c->poison_barrier) return false;
+    const auto mm = std::minmax_element(c->N.begin(), c->N.end());
+    return fx_plan(b, c->R, *mm.first, *mm.second, plan);
+}
+
+dacp_status fx_workspace(dacp_ctx* c, int b, const FxPlan& plan) {
+    const size_t R = static_cast<size_t>(c->R), ctas = R << plan.lg, parts = R * fx_part_sums(b);
+    if (!c->fx_list_d) {
+        TRY(dalloc_t(c, &c->fx_emax_d, R));
+        TRY(dalloc_t(c, &c->fx_status_d, R));
+        TRY(dalloc_t(c, &c->fx_bar_d, R));
+        TRY(dalloc_t(c, &c->fx_list_d, R));
+    }
+    if (ctas > c->fx_ctas) {
+        dfree(c, c->fx_pro_d);
+        c->fx_pro_d = nullptr;
+        c->fx_ctas = 0;
+        TRY(dalloc_t(c, &c->fx_pro_d, ctas));
+        c->fx_ctas = ctas;
+    }
+    if (parts > c->fx_parts) {
+        dfree(c, c->fx_part_d);
+        c->fx_part_d = nullptr;
+        c->fx_parts = 0;
+        TRY(dalloc_t(c, &c->fx_part_d, parts));
+        c->fx_parts = parts;
+    }
+    return DACP_OK;
+}
+
+// Evolution vectors and moment rows of one fixed-point run.
+struct FxRun {
+    int b;
+    const void* psi;                    // start vectors
+    void *pub0, *pub1;                  // two buffers of the batch's vector size
+    double* mom;
+    int mom_rows_fixed, nsteps_override;
+};
+
+// Queue the fixed-point evolution of every realization (longest run first) on the handle's stream;
+// fx_status_d then names those it did not suit. emax: host values, uploaded here.
+dacp_status fx_launch(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std::vector<double>& emax) {
+    TRY(fx_workspace(c, q.b, plan));
+    std::vector<int> order(c->R);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        const int64_t wx = static_cast<int64_t>(q.nsteps_override > 0 ? 1 : c->info[x].ne) << c->N[x];
+        const int64_t wy = static_cast<int64_t>(q.nsteps_override > 0 ? 1 : c->info[y].ne) << c->N[y];
+        return wx > wy;
+    });
+    CK(cudaMemcpyAsync(c->fx_emax_d, emax.data(), sizeof(double) * c->R, cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemcpyAsync(c->fx_list_d, order.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemsetAsync(c->fx_status_d, 0, sizeof(int) * c->R, c->st));
+    CK(cudaMemsetAsync(c->fx_bar_d, 0, sizeof(unsigned) * c->R, c->st));
+    FxArgs a;
+    memset(&a, 0, sizeof(a));
+    a.list = c->fx_list_d;
+    a.real = c->info_d;
+    a.diag = static_cast<const double*>(c->diag_d);
+    a.gam = static_cast<const double*>(c->gam_d);
+    a.psi = static_cast<const double*>(q.psi);
+    a.gflip = c->has_gflip ? c->gflip_d : nullptr;
+    a.emax = c->fx_emax_d;
+    a.pub0 = static_cast<int4*>(q.pub0);
+    a.pub1 = static_cast<int4*>(q.pub1);
+    a.pro = c->fx_pro_d;
+    a.part = c->fx_part_d;
+    a.mom = q.mom;
+    a.bar = c->fx_bar_d;
+    a.status = c->fx_status_d;
+    a.err_flag = c->err_d;
+    a.mom_rows_fixed = q.mom_rows_fixed;
+    a.nsteps_override = q.nsteps_override;
+    CK(launch_evolve_fx(q.b, plan, a, c->R, c->st));
+    c->launches += plan.sync == kFxCounter ? (c->R + plan.groups - 1) / plan.groups : 1;
+    return DACP_OK;
+}
+
+// Wait for a fixed-point run and evolve the realizations it did not suit with the floating-point
+// kernels, one after the other. Leaves the evolution's coefficients on the device if there were any
+// (*redone): the caller restores the filter's.
+dacp_status fx_finish(dacp_ctx* c, const FxRun& q, const std::vector<double>& emax, bool* redone) {
+    std::vector<int> bad(c->R);
+    CK(cudaMemcpyAsync(bad.data(), c->fx_status_d, sizeof(int) * c->R, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    *redone = false;
+    for (int r = 0; r < c->R; ++r) {
+        if (!bad[r]) continue;
+        if (!*redone) TRY(set_evolution_coef(c, emax));
+        *redone = true;
+        const size_t at = static_cast<size_t>(c->info[r].off) * q.b * c->esz;
+        CK(cudaMemcpyAsync(static_cast<char*>(q.pub0) + at, static_cast<const char*>(q.psi) + at,
+                           (static_cast<size_t>(q.b) << c->N[r]) * c->esz, cudaMemcpyDeviceToDevice, c->st));
+        CK(cudaMemsetAsync(c->step_ctr_d, 0, sizeof(int), c->st));
+        StepArgs a = base_args(c);
+        a.bufA = q.pub0;
+        a.bufB = q.pub1;
+        a.mom = q.mom;
+        a.mom_rows_fixed = q.mom_rows_fixed;
+        a.nsteps_override = q.nsteps_override;
+        const int orders = q.nsteps_override > 0 ? q.nsteps_override : c->info[r].ne;
+        for (int k = 0; k < orders; ++k)
+            CK(launch_step(c->prec, q.b, kEvolve, a, c->info[r].item_begin, c->info[r].item_count, c->smem, c->st));
+        c->launches += orders;
+    }
+    if (*redone) CK(cudaStreamSynchronize(c->st));
+    return DACP_OK;
+}
+
 dacp_status set_evolution_coef(dacp_ctx* c, const std::vector<double>& emax) {
     std::vector<double> coef(8 * static_cast<size_t>(c->R), 0.0);
     for (int r = 0; r < c->R; ++r) {
@@ -830,7 +951,7 @@ dacp_status choose_impl(dacp_ctx* c, int n_eigs, double d_ratio, double basis_ra
         if (!c->feats_d) TRY(dalloc_t(c, &c->feats_d, static_cast<size_t>(R) * kFeatures));
         // v = column 0 of psi0, normalised; kept in kA for the KPM run
         CK(launch_extract_col(c->prec, c->b, c->psi0_d, v2, c->Dtot, c->st));
-        c->launches += 3 + 4 * static_cast<int64_t>(steps) + 1 + kpm_moments / 2 + 2;
+        c->launches += 3 + 4 * static_cast<int64_t>(steps) + 1 + 2;
         CK(launch_normalize(c->prec, 1, c->items_d, c->info_d, ni, v2, v2, 0, c->part_d, c->real_done_d,
                             c->norms_d, v1, kA, c->st));
         // Lanczos: w = H v - beta v_prev; alpha = <w, v>; w -= alpha v; beta = |w|
@@ -873,15 +994,24 @@ dacp_status choose_impl(dacp_ctx* c, int n_eigs, double d_ratio, double basis_ra
         if (c->emax_rule == 1) CK(cudaMemcpyAsync(em1.data(), emax1_d, R * 8, cudaMemcpyDeviceToHost, c->st));
         CK(cudaStreamSynchronize(c->st));
         // KPM moments of the normalised start vector under G = H / E_max
-        TRY(set_evolution_coef(c, em));
-        StepArgs a = base_args(c);
-        a.bufA = kA;
-        a.bufB = kB;
-        a.mom = kp;
-        a.mom_rows_fixed = kpm_moments;
-        a.nsteps_override = kpm_moments / 2;
-        CK(cudaMemsetAsync(c->step_ctr_d, 0, sizeof(int), c->st));
-        for (int k = 0; k < kpm_moments / 2; ++k) CK(launch_step(c->prec, 1, kEvolve, a, 0, ni, c->smem, c->st));
+        FxPlan plan;
+        if (fx_usable(c, 1, &plan)) {
+            const FxRun q{1, kA, kB, v0, kp, kpm_moments, kpm_moments / 2};
+            bool redone = false;
+            TRY(fx_launch(c, plan, q, em));
+            TRY(fx_finish(c, q, em, &redone));
+        } else {
+            c->launches += kpm_moments / 2;
+            TRY(set_evolution_coef(c, em));
+            StepArgs a = base_args(c);
+            a.bufA = kA;
+            a.bufB = kB;
+            a.mom = kp;
+            a.mom_rows_fixed = kpm_moments;
+            a.nsteps_override = kpm_moments / 2;
+            CK(cudaMemsetAsync(c->step_ctr_d, 0, sizeof(int), c->st));
+            for (int k = 0; k < kpm_moments / 2; ++k) CK(launch_step(c->prec, 1, kEvolve, a, 0, ni, c->smem, c->st));
+        }
         CK(launch_features(R, c->info_d, c->J_d, c->h_d, c->g64_d, kp, kpm_moments, n_eigs, c->feats_d, c->st));
         if (net) {
             int64_t nl = 0;
@@ -995,10 +1125,19 @@ dacp_status dacp_basis_moments(dacp_handle c) {
     const size_t vec_bytes = static_cast<size_t>(c->Dtot) * c->b * c->esz;
     int maxE = 0;
     for (int r = 0; r < c->R; ++r) maxE = std::max(maxE, c->info[r].ne);
-    TRY(set_evolution_coef(c, c->emax));
-    CK(cudaEventRecord(c->ev[2], c->st));
-    CK(cudaMemcpyAsync(c->A_d, c->psiE_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
-    TRY(run_orders(c, false, maxE));
+    FxPlan plan;
+    bool coef = true;
+    if (fx_usable(c, c->b, &plan)) {
+        const FxRun q{c->b, c->psiE_d, c->A_d, c->B_d, c->mom_d, 0, 0};
+        CK(cudaEventRecord(c->ev[2], c->st));
+        TRY(fx_launch(c, plan, q, c->emax));
+        TRY(fx_finish(c, q, c->emax, &coef));
+    } else {
+        TRY(set_evolution_coef(c, c->emax));
+        CK(cudaEventRecord(c->ev[2], c->st));
+        CK(cudaMemcpyAsync(c->A_d, c->psiE_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
+        TRY(run_orders(c, false, maxE));
+    }
     CK(cudaEventRecord(c->ev[3], c->st));
     CK(cudaStreamSynchronize(c->st));
     TRY(check_device_flag(c));
@@ -1006,7 +1145,7 @@ dacp_status dacp_basis_moments(dacp_handle c) {
     cudaEventElapsedTime(&ms, c->ev[2], c->ev[3]);
     c->t_ms[1] = ms;
     // restore the filter coefficients for a later dacp_filter
-    TRY(apply_params(c));
+    if (coef) TRY(apply_params(c));
     c->state = 3;
     return DACP_OK;
 }
@@ -1446,6 +1585,7 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
     };
 
     std::thread th;
+    bool coef = true;                   // the device holds the evolution's coefficients
     auto push = [&](const std::vector<int>& order, int from, int to) -> dacp_status {
         cudaEvent_t ev = nullptr;
         CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -1478,10 +1618,18 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
             return DACP_OK;
         };
         const size_t vec_bytes = static_cast<size_t>(c->Dtot) * c->b * c->esz;
-        TRY(set_evolution_coef(c, c->emax));
-        CK(cudaEventRecord(c->ev[2], c->st));
-        CK(cudaMemcpyAsync(c->A_d, c->psiE_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
-        TRY(run_orders(c, false, maxE, after));
+        FxPlan plan;
+        if (fx_usable(c, b, &plan)) {
+            const FxRun q{b, c->psiE_d, c->A_d, c->B_d, c->mom_d, 0, 0};
+            CK(cudaEventRecord(c->ev[2], c->st));
+            TRY(fx_launch(c, plan, q, c->emax));
+            TRY(fx_finish(c, q, c->emax, &coef));
+        } else {
+            TRY(set_evolution_coef(c, c->emax));
+            CK(cudaEventRecord(c->ev[2], c->st));
+            CK(cudaMemcpyAsync(c->A_d, c->psiE_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
+            TRY(run_orders(c, false, maxE, after));
+        }
         CK(cudaEventRecord(c->ev[3], c->st));
         if (dispatched < R) TRY(push(order, dispatched, R));
         return DACP_OK;
@@ -1512,7 +1660,7 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
     ws_free(c, w);
     if (st != DACP_OK) return st;
     // restore the filter coefficients for a later dacp_filter
-    TRY(apply_params(c));
+    if (coef) TRY(apply_params(c));
     c->state = 3;
     return DACP_OK;
 }
@@ -1845,6 +1993,12 @@ dacp_status dacp_eigenvectors(dacp_handle c, int r, int n_eigs, double window, d
         }
         StepArgs a = base_args(c);
         const int i0 = c->info[r].item_begin, ni = c->info[r].item_count;
+        // the replay's moment rows go to a scratch array: the handle keeps those of its evolution
+        const int64_t bb = static_cast<int64_t>(b) * b;
+        double* rows = nullptr;
+        TRY(dalloc_t(c, &rows, static_cast<size_t>(2 * c->info[r].ne * bb)));
+        z.tmp.push_back(rows);
+        a.mom = rows - c->info[r].mom_off * bb;
         for (int k = 0; next < Ln; ++k) {
             CK(launch_step(c->prec, b, kEvolve, a, i0, ni, c->smem, c->st));   // w_{k+1}
             c->launches += 1;
@@ -1865,7 +2019,7 @@ dacp_status dacp_eigenvectors(dacp_handle c, int r, int n_eigs, double window, d
     dacp_status s = run();
     ritz_free(c, z);
     if (s != DACP_OK) return s;
-    // restore the filter coefficients; the moments of r were rewritten with the same values
+    // restore the filter coefficients
     TRY(apply_params(c));
     c->state = 3;
     return DACP_OK;

@@ -3,8 +3,8 @@
 // Some callers cannot call cudaMalloc: engines whose device memory all
 // belongs to their own pool or arena, and latency-critical loops that forbid
 // allocator calls. For them this entry point runs the float64 evolution
-// stencil (H.v fused with the Chebyshev recurrence and the moment sums) for
-// one realization without allocating anything: its working vectors,
+// (H.v fused with the Chebyshev recurrence and the moment sums, resident in
+// shared memory) for one realization without allocating anything: its working vectors,
 // diagonal, couplings, partial sums and counters live in one file-scope
 // device array, and the caller passes only the input vector and the output
 // moments. The call copies its small host inputs into the array on the
@@ -45,7 +45,9 @@ constexpr int64_t kRegPart = kRegCoef + 32;               // per-tile moment par
 constexpr int64_t kRegInfo = kRegPart + 2 * kNaMaxItems + 32;   // RealInfo
 constexpr int64_t kRegItems = kRegInfo + 32;              // Item[kNaMaxItems]
 constexpr int64_t kRegCount = kRegItems + kNaMaxItems + 32;     // counters (unsigned / int)
-constexpr int64_t kNaTotal = kRegCount + 32;
+constexpr int64_t kRegEmax = kRegCount + 32;              // E_max
+constexpr int64_t kRegPro = kRegEmax + 32;                // scale exchange of the resident evolution
+constexpr int64_t kNaTotal = kRegPro + (2 << kFxMaxLg);
 
 static_assert(sizeof(RealInfo) <= 32 * sizeof(double), "RealInfo region too small");
 static_assert(sizeof(Item) * kNaMaxItems <= (kNaMaxItems + 32) * sizeof(double), "Item region too small");
@@ -121,7 +123,7 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
     // order 0: w_1 = G psi; then w_{k+1} = 2 G w_k - w_{k-1}, G = H / E_max
     const double coef[8] = {1.0 / emax, 0.0, 0.0, 2.0 / emax, -1.0, 0.0, 0.0, 0.0};
 
-    unsigned* counters = reinterpret_cast<unsigned*>(base + kRegCount);   // real_done, launch_done, step, err, bar[2]
+    unsigned* counters = reinterpret_cast<unsigned*>(base + kRegCount);   // real_done, launch_done, step, err, bar[2], list, status
     auto ok = [](cudaError_t e) { return e == cudaSuccess; };
     // Calls share the array and it keeps the last call's contents: everything
     // read before it is written is set again here, counters cleared to zero.
@@ -131,13 +133,46 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
                 ok(cudaMemcpyAsync(base + kRegH, hp, sizeof(hp), cudaMemcpyHostToDevice, st)) &&
                 ok(cudaMemcpyAsync(base + kRegGam, gp, sizeof(gp), cudaMemcpyHostToDevice, st)) &&
                 ok(cudaMemcpyAsync(base + kRegCoef, coef, sizeof(coef), cudaMemcpyHostToDevice, st)) &&
-                ok(cudaMemsetAsync(counters, 0, 8 * sizeof(unsigned), st)) &&
-                ok(cudaMemcpyAsync(base + kRegA, psi_dev, sizeof(double) * D, cudaMemcpyDeviceToDevice, st));
+                ok(cudaMemcpyAsync(base + kRegEmax, &emax, sizeof(emax), cudaMemcpyHostToDevice, st)) &&
+                ok(cudaMemsetAsync(counters, 0, 8 * sizeof(unsigned), st));
     if (!good) return DACP_ERR_CUDA;
     const RealInfo* info_d = reinterpret_cast<const RealInfo*>(base + kRegInfo);
     if (launch_diag(kPrecF64, info_d, 0, N, base + kRegJ, base + kRegH, base + kRegDiag, st) != cudaSuccess)
         return DACP_ERR_CUDA;
 
+    // the resident fixed-point evolution; what it does not suit (status word set) runs in floating point
+    const int n = 2 * n_orders;
+    FxPlan plan;
+    if (fx_plan(1, 1, N, N, &plan)) {
+        FxArgs f;
+        memset(&f, 0, sizeof(f));
+        f.list = reinterpret_cast<const int*>(counters + 6);            // 0: the one realization
+        f.real = info_d;
+        f.diag = base + kRegDiag;
+        f.gam = base + kRegGam;
+        f.psi = psi_dev;
+        f.emax = base + kRegEmax;
+        f.pub0 = reinterpret_cast<int4*>(base + kRegA);
+        f.pub1 = reinterpret_cast<int4*>(base + kRegB);
+        f.pro = reinterpret_cast<float4*>(base + kRegPro);
+        f.part = reinterpret_cast<longlong2*>(base + kRegPart);
+        f.mom = mu_dev;
+        f.bar = counters + 4;
+        f.status = reinterpret_cast<int*>(counters + 7);
+        f.err_flag = reinterpret_cast<int*>(counters + 3);
+        if (launch_evolve_fx(1, plan, f, 1, st) != cudaSuccess) return DACP_ERR_CUDA;
+        noalloc_moments_from_products<<<(n + 255) / 256, 256, 0, st>>>(mu_dev, n);
+        unsigned words[5];                   // error flag .. status
+        if (cudaGetLastError() != cudaSuccess ||
+            !ok(cudaMemcpyAsync(words, counters + 3, sizeof(words), cudaMemcpyDeviceToHost, st)) ||
+            !ok(cudaStreamSynchronize(st)))
+            return DACP_ERR_CUDA;
+        if (words[0]) return DACP_ERR_TIMEOUT;
+        if (!words[4]) return DACP_OK;
+    }
+    if (!ok(cudaMemsetAsync(counters + 4, 0, sizeof(unsigned), st)) ||
+        !ok(cudaMemcpyAsync(base + kRegA, psi_dev, sizeof(double) * D, cudaMemcpyDeviceToDevice, st)))
+        return DACP_ERR_CUDA;
     StepArgs a;
     memset(&a, 0, sizeof(a));
     a.items = reinterpret_cast<const Item*>(base + kRegItems);
@@ -159,7 +194,6 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
     const int smem = (1 << R.tbits) * static_cast<int>(sizeof(double));
     for (int k = 0; k < n_orders; ++k)
         if (launch_step(kPrecF64, 1, kEvolve, a, 0, R.item_count, smem, st) != cudaSuccess) return DACP_ERR_CUDA;
-    const int n = 2 * n_orders;
     noalloc_moments_from_products<<<(n + 255) / 256, 256, 0, st>>>(mu_dev, n);
     if (cudaGetLastError() != cudaSuccess) return DACP_ERR_CUDA;
     int err = 0;

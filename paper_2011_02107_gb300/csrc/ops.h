@@ -35,6 +35,31 @@ cudaError_t launch_normalize(int prec, int b, const Item* items, const RealInfo*
                              double* norms, void* dst, void* dst2, cudaStream_t st);
 cudaError_t launch_extract_col(int prec, int b, const void* src, void* dst, int64_t states, cudaStream_t st);
 
+// resident.cu: the float64 evolution with both vectors in shared memory, in fixed point
+constexpr int kFxThreads = 512;     // threads of the recurrence per CTA
+constexpr int kFxMaxLg = 7;         // up to 2^7 CTAs per realization
+enum FxSync { kFxAlone = 0, kFxCluster = 1, kFxCounter = 2 };
+struct FxPlan {
+    int lg, sync, u, threads, slots_max, smem, groups;
+};
+struct FxArgs {
+    const int* list;                // realizations, one group of 2^lg CTAs each
+    const RealInfo* real;
+    const double *diag, *gam, *psi;
+    const double *gflip, *emax;     // [R]; gflip nullptr: none
+    int4 *pub0, *pub1;              // published vectors (as many bytes as a float64 vector of the batch)
+    float4* pro;                    // [groups][2^lg] scale exchange
+    longlong2* part;                // [groups][4][sums] moment sums in flight: x 2^24 + y
+    double* mom;
+    unsigned* bar;                  // [groups] barrier counters, zero (kFxCounter)
+    int* status;                    // [R] set to 1: evolve this realization in floating point
+    int* err_flag;
+    int lg, sync, slots_max, mom_rows_fixed, nsteps_override;
+};
+int fx_part_sums(int b);            // elements of FxArgs::part per group
+bool fx_plan(int b, int count, int minN, int maxN, FxPlan* p);
+cudaError_t launch_evolve_fx(int b, const FxPlan& p, const FxArgs& a, int count, cudaStream_t st);
+
 // subspace.cu
 cudaError_t launch_orders(int L, double a_r, int* orders, cudaStream_t st);
 cudaError_t launch_moments(const double* P, int rows, int b, double emax, double* mus, double* nus, int* bad,

@@ -1,0 +1,102 @@
+"""The resident evolution (csrc/resident.cu) against the oracle's directly recorded moments.
+
+One case per way a realization is laid out: tiles below one CTA's least size, one CTA, clusters of
+2 to 8 CTAs, CTAs on a counter barrier; every block size; with and without the global flip; and the
+start vectors and couplings the fixed-point form hands to the floating-point kernels.
+
+Tolerance, from the recurrence: an order adds a rounding error of norm at most (N + 8) u to w_k
+(N + 2 products and sums, one store), u = 2^-53 for float64 and 2^-44 for double-float; an error made
+at order j reaches order k through U_{k-j}(G), of norm at most k - j + 1; and mu_j comes from products
+of two such vectors, doubled. With n orders that is at most 4 (N + 8) u n^2; the reference adds as much.
+"""
+
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import dacp as DA
+from oracle import hamiltonian as Hm
+
+pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+P = pytest.importorskip("paper_2011_02107_gb300")
+
+
+def _bound(m):
+    return float(np.abs(Hm.diagonal(m)).max() + np.abs(m["gamma"]).sum() + abs(m.get("gflip", 0.0)))
+
+
+def _check(models, psis, b, orders, prec, unit, emax=None):
+    emax = np.array([_bound(m) for m in models]) if emax is None else emax
+    n = max(1, int(orders * 0.2 / np.pi))                 # a = 0.2 E_max: k_n = floor(n pi / 0.2)
+    d = P.Dacp(models, psis, block_b=b, precision=prec)
+    try:
+        d.set_params(emax, 0.2 * emax, 0, n)              # K = 0: psi_E is the start block, normalised
+        d.filter()
+        d.basis_moments()
+        kn = d.params()["kn"]
+        for r, m in enumerate(models):
+            mu = d.moments(r)
+            ref, _ = DA.chebyshev_moments(m, d.filtered(r), emax[r], mu.shape[0] - 1)
+            ref = 0.5 * (ref + ref.transpose(0, 2, 1))
+            tol = 8 * (m["N"] + 8) * unit * (kn[r] + 2) ** 2
+            err = np.abs(mu - ref).max()
+            assert err <= tol, (r, m["N"], err, tol)
+    finally:
+        d.close()
+
+
+def _flip(m, c):
+    return dict(m, gflip=c)
+
+
+PRECS = [("fp64", P.DACP_FP64, 2.0 ** -53)]
+
+
+@pytest.mark.parametrize("name,prec,unit", PRECS)
+@pytest.mark.parametrize("flip", [False, True])
+@pytest.mark.parametrize("b", [1, 2, 4])
+@pytest.mark.parametrize("Ns", [(1, 2, 3, 4), (5, 9, 12, 7, 10), (6, 6), (13,), (8,)])
+def test_resident_evolution_on_small_batches(Ns, b, flip, name, prec, unit):
+    models = [W.random_model(N, seed=70 + i) for i, N in enumerate(Ns)]
+    if flip:
+        models = [_flip(m, 0.41 * (-1) ** i) for i, m in enumerate(models)]
+    psis = [W.start_vectors(N, b, seed=3, r=i) for i, N in enumerate(Ns)]
+    _check(models, psis, b, 40, prec, unit)
+
+
+@pytest.mark.parametrize("name,prec,unit", PRECS)
+@pytest.mark.parametrize("N,b,count", [(14, 4, 2), (13, 4, 40), (16, 2, 1), (16, 4, 1), (15, 1, 1)])
+def test_resident_evolution_over_many_ctas(N, b, count, name, prec, unit):
+    models = [_flip(W.spin_glass_shard(N, seed=5 + r), 0.3) for r in range(count)]
+    psis = [W.start_vectors(N, b, seed=4, r=r) for r in range(count)]
+    _check(models, psis, b, 24, prec, unit)
+
+
+@pytest.mark.parametrize("name,prec,unit", PRECS)
+@pytest.mark.parametrize("N", [6, 11])
+def test_start_vectors_of_one_state_and_of_uneven_size(N, name, prec, unit):
+    """A basis state (all the norm in one element), a smooth vector with elements down to 1e-30, and an
+    ordinary block in one batch: those the fixed point does not suit go through the other kernels."""
+    one = np.zeros((1 << N, 2))
+    one[3, 0] = one[5, 1] = 1.0
+    decay = np.exp(-np.arange(1 << N) * 69.0 / (1 << N))[:, None] * np.array([[1.0, -1.0]])
+    decay[::2, 1] *= 0.5
+    models = [W.random_model(N, seed=80 + i) for i in range(3)]
+    _check(models, [one, W.start_vectors(N, 2, seed=6), decay], 2, 30, prec, unit)
+
+
+@pytest.mark.parametrize("name,prec,unit", PRECS)
+def test_bound_far_below_the_radius_is_reported_as_before(name, prec, unit):
+    """Coefficients beyond the limbs, and vectors that outgrow the fixed point, end as DACP_ERR_NUMERIC."""
+    m = W.chain(9)
+    for shrink in (0.02, 0.6):
+        em = shrink * np.abs(np.linalg.eigvalsh(Hm.dense_h(m))).max()
+        d = P.Dacp([m, m], [W.start_vectors(9, 2, seed=0, r=r) for r in range(2)], block_b=2, precision=prec)
+        try:
+            d.set_params(em, 0.3 * em, 0, 8)
+            d.filter()
+            d.basis_moments()
+            assert (d.central_eigs(4)[1] == -4).all()
+        finally:
+            d.close()
