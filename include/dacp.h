@@ -209,7 +209,10 @@ dacp_status dacp_filter(dacp_handle hd);
  * memory of up to 128 CTAs (2^18 states at b = 4) evolve them there in 59-bit
  * fixed point, which is at least as accurate as float64 vectors; realizations
  * it does not suit (an element above 16 times the root mean square, or E_max
- * not a bound) and all other handles use float64 vectors in device memory.
+ * not a bound) use float64 vectors in device memory. DACP_DF32 handles with
+ * b = 4, no pair couplings and uniform tiles of 2^10 or 2^11 states, at most 8
+ * to a realization, keep them in the shared memory of one cluster in launch
+ * mode 0; vectors and moments have the bits of the per-order launch.
  * Errors: DACP_ERR_NUMERIC when a realization's |mu_j| exceeds mu_0 (E_max
  * was not a bound) -- reported per realization by dacp_central_eigs.
  */
@@ -367,8 +370,8 @@ dacp_status dacp_autotune(dacp_handle hd, int orders, int* tile_bytes_out);
  * of two, 1 KB to 128 KB). Mode 2 needs (1 + recurrence terms) tiles plus the
  * tile's diagonal in shared memory, so tiles above 64 KB are refused there
  * (DACP_ERR_ARG), as is mode 2 on float64 or double-float vectors. Setting
- * resets filter and moment results. An evolution resident in shared memory
- * (see dacp_basis_moments) does not depend on mode and tile size.
+ * resets filter and moment results. The resident evolution of DACP_FP64
+ * handles (see dacp_basis_moments) does not depend on mode and tile size.
  */
 dacp_status dacp_set_launch(dacp_handle hd, int mode, int tile_bytes);
 dacp_status dacp_get_launch(dacp_handle hd, int* mode, int* tile_bytes);

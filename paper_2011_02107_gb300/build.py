@@ -16,7 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libdacp.so")
-SOURCES = ["stencil.cu", "resident.cu", "subspace.cu", "params.cu", "mlp.cu", "api.cu", "noalloc.cu"]
+SOURCES = ["stencil.cu", "resident.cu", "resident_df.cu", "subspace.cu", "params.cu", "mlp.cu", "api.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr"]

@@ -130,6 +130,9 @@ struct dacp_ctx {
     float4* fx_pro_d = nullptr;
     longlong2* fx_part_d = nullptr;
     size_t fx_ctas = 0, fx_parts = 0;
+    double* df_part_d = nullptr;        // double-float resident evolution (resident_df.cu): sums in flight
+    size_t df_parts = 0;
+    std::vector<cudaStream_t> df_st;    // streams its groups run on beside each other (dacp_solve)
 
     // parameters
     std::vector<double> emax, a;
@@ -532,14 +535,20 @@ bool fx_usable(const dacp_ctx* c, int b, FxPlan* plan) {
     return fx_plan(b, c->R, *mm.first, *mm.second, plan);
 }
 
+// Per-realization arrays of a resident launch.
+dacp_status resident_lists(dacp_ctx* c) {
+    const size_t R = static_cast<size_t>(c->R);
+    if (c->fx_list_d) return DACP_OK;
+    TRY(dalloc_t(c, &c->fx_emax_d, R));
+    TRY(dalloc_t(c, &c->fx_status_d, R));
+    TRY(dalloc_t(c, &c->fx_bar_d, R));
+    TRY(dalloc_t(c, &c->fx_list_d, R));
+    return DACP_OK;
+}
+
 dacp_status fx_workspace(dacp_ctx* c, int b, const FxPlan& plan) {
     const size_t R = static_cast<size_t>(c->R), ctas = R << plan.lg, parts = R * fx_part_sums(b);
-    if (!c->fx_list_d) {
-        TRY(dalloc_t(c, &c->fx_emax_d, R));
-        TRY(dalloc_t(c, &c->fx_status_d, R));
-        TRY(dalloc_t(c, &c->fx_bar_d, R));
-        TRY(dalloc_t(c, &c->fx_list_d, R));
-    }
+    TRY(resident_lists(c));
     if (ctas > c->fx_ctas) {
         dfree(c, c->fx_pro_d);
         c->fx_pro_d = nullptr;
@@ -636,6 +645,72 @@ dacp_status fx_finish(dacp_ctx* c, const FxRun& q, const std::vector<double>& em
     return DACP_OK;
 }
 
+// Whether the evolution of launch mode 0 runs as resident double-float clusters, one CTA per tile of the
+// per-order launch (whose bits it keeps). Clusters of up to 4 CTAs win at every batch size: 4.11 against 8.00 ms
+// for 361 orders of 36 13-spin sectors, 61.4 against 64.8 ms of 512. Of 8 CTAs only 15 fit the GPU (120 of
+// 152 SMs), so there the per-order launch is ahead once they do not all run at once: 79.1 against 65.2 ms
+// for 256 14-spin shards.
+bool df_resident_usable(const dacp_ctx* c) {
+    if (c->prec != kPrecDF32 || c->b != 4 || c->has_pairs || c->launch_mode != 0) return false;
+    const int max_N = *std::max_element(c->N.begin(), c->N.end());
+    return df4_resident_fits(c->tb_uniform, max_N) && (max_N - c->tb_uniform < 3 || c->R <= 15);
+}
+
+// Queue the resident double-float evolution of the realizations order[0 .. R), group by group: group g is
+// order[from[g] .. from[g + 1]) (from ends with R) and runs on stream st[g], in rising group order where
+// SMs are short and with the longest runs of a group first. psi_E, the two recurrence buffers and the moment
+// rows are the handle's.
+dacp_status df_resident_launch(dacp_ctx* c, const std::vector<int>& order, const std::vector<int>& from,
+                               const std::vector<cudaStream_t>& st) {
+    TRY(resident_lists(c));
+    DfResArgs a;
+    memset(&a, 0, sizeof(a));
+    for (a.lg = 0; c->tb_uniform + a.lg < *std::max_element(c->N.begin(), c->N.end());) ++a.lg;
+    const size_t parts = (static_cast<size_t>(c->R) << a.lg) * kDfPartSums;
+    if (parts > c->df_parts) {
+        dfree(c, c->df_part_d);
+        c->df_part_d = nullptr;
+        c->df_parts = 0;
+        TRY(dalloc_t(c, &c->df_part_d, parts));
+        c->df_parts = parts;
+    }
+    const int ng = static_cast<int>(from.size()) - 1;
+    std::vector<int> list(order);
+    for (int g = 0; g < ng; ++g)
+        std::stable_sort(list.begin() + from[g], list.begin() + from[g + 1],
+                         [&](int x, int y) { return c->info[x].ne > c->info[y].ne; });
+    CK(cudaMemcpyAsync(c->fx_emax_d, c->emax.data(), sizeof(double) * c->R, cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemcpyAsync(c->fx_list_d, list.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
+    CK(cudaEventRecord(c->ev[2], c->st));            // also the start of T_E
+    a.real = c->info_d;
+    a.diag = static_cast<const df32*>(c->diag_d);
+    a.gam = static_cast<const df32*>(c->gam_d);
+    a.gflip = c->has_gflip ? c->gflip_d : nullptr;
+    a.emax = c->fx_emax_d;
+    a.psi = c->psiE_d;
+    a.pub0 = static_cast<ulonglong2*>(c->A_d);
+    a.pub1 = static_cast<ulonglong2*>(c->B_d);
+    a.mom = c->mom_d;
+    for (int g = 0; g < ng; ++g) {
+        if (st[g] != c->st) CK(cudaStreamWaitEvent(st[g], c->ev[2], 0));
+        a.list = c->fx_list_d + from[g];
+        a.part = c->df_part_d + (static_cast<size_t>(from[g]) << a.lg) * kDfPartSums;
+        CK(launch_evolve_df4_resident(c->tb_uniform, a, from[g + 1] - from[g], st[g]));
+        c->launches += 1;
+    }
+    return DACP_OK;
+}
+
+// `count` streams beside the handle's own.
+dacp_status df_resident_streams(dacp_ctx* c, size_t count) {
+    while (c->df_st.size() < count) {
+        cudaStream_t s = nullptr;
+        CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+        c->df_st.push_back(s);
+    }
+    return DACP_OK;
+}
+
 dacp_status set_evolution_coef(dacp_ctx* c, const std::vector<double>& emax) {
     std::vector<double> coef(8 * static_cast<size_t>(c->R), 0.0);
     for (int r = 0; r < c->R; ++r) {
@@ -674,6 +749,10 @@ void dacp_destroy(dacp_handle c) {
     cudaSetDevice(c->device);
     if (c->st) cudaStreamSynchronize(c->st);
     if (c->st2) cudaStreamSynchronize(c->st2);
+    for (cudaStream_t s : c->df_st) {
+        cudaStreamSynchronize(s);
+        cudaStreamDestroy(s);
+    }
     free_lanes(c);
     if (c->gf.exec) cudaGraphExecDestroy(c->gf.exec);
     if (c->ge.exec) cudaGraphExecDestroy(c->ge.exec);
@@ -1132,6 +1211,11 @@ dacp_status dacp_basis_moments(dacp_handle c) {
         CK(cudaEventRecord(c->ev[2], c->st));
         TRY(fx_launch(c, plan, q, c->emax));
         TRY(fx_finish(c, q, c->emax, &coef));
+    } else if (df_resident_usable(c)) {
+        std::vector<int> order(c->R);
+        std::iota(order.begin(), order.end(), 0);
+        TRY(df_resident_launch(c, order, {0, c->R}, {c->st}));
+        coef = false;
     } else {
         TRY(set_evolution_coef(c, c->emax));
         CK(cudaEventRecord(c->ev[2], c->st));
@@ -1586,11 +1670,11 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
 
     std::thread th;
     bool coef = true;                   // the device holds the evolution's coefficients
-    auto push = [&](const std::vector<int>& order, int from, int to) -> dacp_status {
+    auto push = [&](const std::vector<int>& order, int from, int to, cudaStream_t st) -> dacp_status {
         cudaEvent_t ev = nullptr;
         CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
         events.push_back(ev);
-        CK(cudaEventRecord(ev, c->st));
+        CK(cudaEventRecord(ev, st));
         Job j;
         j.idx.assign(order.begin() + from, order.begin() + to);
         j.ev = ev;
@@ -1609,10 +1693,10 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return c->info[x].ne < c->info[y].ne; });
         th = std::thread(worker);
         int dispatched = 0, complete = 0;
-        auto after = [&](int done) -> dacp_status {
+        std::function<dacp_status(int)> after = [&](int done) -> dacp_status {
             while (complete < R && c->info[order[complete]].ne <= done) ++complete;
             if (complete - dispatched >= chunk) {
-                TRY(push(order, dispatched, complete));
+                TRY(push(order, dispatched, complete, c->st));
                 dispatched = complete;
             }
             return DACP_OK;
@@ -1624,6 +1708,28 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
             CK(cudaEventRecord(c->ev[2], c->st));
             TRY(fx_launch(c, plan, q, c->emax));
             TRY(fx_finish(c, q, c->emax, &coef));
+        } else if (df_resident_usable(c)) {
+            // the groups that the per-order launch would hand over (their composition sets the padding of
+            // the batched solves); each runs on a stream of its own, so that a group's solves start when
+            // its evolution ends while the clusters of later groups take the SMs that become free
+            std::vector<int> from(1, 0);
+            after = [&](int done) -> dacp_status {
+                while (complete < R && c->info[order[complete]].ne <= done) ++complete;
+                if (complete - from.back() >= chunk) from.push_back(complete);
+                return DACP_OK;
+            };
+            for (int done = kGraphOrders; done <= maxE; done += kGraphOrders) TRY(after(done));
+            for (int done = maxE - maxE % kGraphOrders + 1; done <= maxE; ++done) TRY(after(done));
+            if (from.back() < R) from.push_back(R);
+            const size_t ng = from.size() - 1;
+            TRY(df_resident_streams(c, ng - 1));
+            std::vector<cudaStream_t> st(c->df_st.begin(), c->df_st.begin() + (ng - 1));
+            st.insert(st.begin(), c->st);
+            TRY(df_resident_launch(c, order, from, st));
+            coef = false;
+            dispatched = R;
+            for (size_t g = 0; g < ng; ++g) TRY(push(order, from[g], from[g + 1], st[g]));
+            for (size_t g = 1; g < ng; ++g) CK(cudaStreamWaitEvent(c->st, events[g], 0));
         } else {
             TRY(set_evolution_coef(c, c->emax));
             CK(cudaEventRecord(c->ev[2], c->st));
@@ -1631,7 +1737,7 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
             TRY(run_orders(c, false, maxE, after));
         }
         CK(cudaEventRecord(c->ev[3], c->st));
-        if (dispatched < R) TRY(push(order, dispatched, R));
+        if (dispatched < R) TRY(push(order, dispatched, R, c->st));
         return DACP_OK;
     };
     dacp_status st = run();
@@ -1647,6 +1753,7 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
     }
     cudaStreamSynchronize(s2.st);
     cudaStreamSynchronize(c->st);
+    for (cudaStream_t s : c->df_st) cudaStreamSynchronize(s);
     if (st == DACP_OK) st = check_device_flag(c);
     if (st == DACP_OK) {
         float te = 0.f, td = 0.f;

@@ -9,6 +9,7 @@
 namespace dacp {
 
 // stencil.cu
+cudaError_t grow_smem_attr(const void* func, int smem);     // a kernel's dynamic shared memory, only upwards
 cudaError_t prepare_step(int prec, int b, int smem);
 cudaError_t launch_persistent(int prec, int b, int seq, const StepArgs& a, int n_items, int orders, int smem,
                               cudaStream_t st, int* grid_out);
@@ -59,6 +60,22 @@ struct FxArgs {
 int fx_part_sums(int b);            // elements of FxArgs::part per group
 bool fx_plan(int b, int count, int minN, int maxN, FxPlan* p);
 cudaError_t launch_evolve_fx(int b, const FxPlan& p, const FxArgs& a, int count, cudaStream_t st);
+
+// resident_df.cu: the double-float b = 4 evolution with both vectors in shared memory
+struct DfResArgs {
+    const int* list;                // realizations, one cluster of 2^lg CTAs each
+    const RealInfo* real;
+    const df32 *diag, *gam;
+    const double *gflip, *emax;     // [R]; gflip nullptr: none
+    const void* psi;
+    ulonglong2 *pub0, *pub1;        // published vectors, as a vector of the batch
+    double* part;                   // [clusters][4][2^lg][32] moment sums in flight
+    double* mom;
+    int lg;
+};
+constexpr int kDfPartSums = 4 * 32; // doubles of DfResArgs::part per CTA
+bool df4_resident_fits(int tbits_uniform, int max_N);
+cudaError_t launch_evolve_df4_resident(int tbits, const DfResArgs& a, int count, cudaStream_t st);
 
 // subspace.cu
 cudaError_t launch_orders(int L, double a_r, int* orders, cudaStream_t st);

@@ -34,6 +34,7 @@
 
 #include "common.cuh"
 #include "ops.h"
+#include "warp.cuh"
 
 namespace dacp {
 
@@ -75,26 +76,6 @@ struct FxMom {
         return (hh + ((mm + (int64_t(1) << 28)) >> 29) + half) >> shift;
     }
 };
-
-// Sum V = 2^v values per lane over the lanes that differ in the bits >= OMIN; lane L keeps value
-// L / (32 / V) (see warp_reduce_scatter in stencil.cu).
-template <int V, int OMIN>
-__device__ __forceinline__ int64_t fx_reduce_scatter(int64_t (&x)[V], const int lane) {
-#pragma unroll
-    for (int half = V / 2, o = 16; half >= 1; half >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < half; ++i) {
-            const int64_t send = up ? x[i] : x[i + half];
-            const int64_t keep = up ? x[i + half] : x[i];
-            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    int64_t v = x[0];
-#pragma unroll
-    for (int o = 16 / V; o >= OMIN; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // Barrier of the realization's group: the CTA alone, a cluster, or CTAs of a cooperative launch
 // on a counter (bounded: false when one second passes, and then at every CTA of the group).
@@ -494,18 +475,18 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
                 int64_t v[16];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) v[e] = e < 10 ? ms[e].fold(msh, half) : 0;
-                const int64_t s = fx_reduce_scatter<16, 2>(v, lane);
+                const int64_t s = warp_reduce_scatter<16, 2>(v, lane);
                 const int e = lane >> 1;
                 if (e < 10) red_s[k % kFxRedRing][warp][(lane & 1) * 10 + e] = s;
             } else if constexpr (B == 2) {
                 int64_t v[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) v[e] = e < 6 ? ms[e].fold(msh, half) : 0;
-                const int64_t s = fx_reduce_scatter<8, 1>(v, lane);
+                const int64_t s = warp_reduce_scatter<8>(v, lane);
                 if ((lane & 3) == 0 && (lane >> 2) < 6) red_s[k % kFxRedRing][warp][lane >> 2] = s;
             } else {
                 int64_t v[2] = {ms[0].fold(msh, half), ms[1].fold(msh, half)};
-                const int64_t s = fx_reduce_scatter<2, 1>(v, lane);
+                const int64_t s = warp_reduce_scatter<2>(v, lane);
                 if ((lane & 15) == 0) red_s[k % kFxRedRing][warp][lane >> 4] = s;
             }
         }

@@ -33,6 +33,7 @@
 
 #include "common.cuh"
 #include "ops.h"
+#include "warp.cuh"
 
 namespace dacp {
 
@@ -85,40 +86,6 @@ __device__ __forceinline__ void load_vals_ro(const T* __restrict__ p, T (&v)[B])
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ __forceinline__ df32 shfl_xor_df(df32 v, int o) {
-    return df32(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
-}
-
-// Sums V = 2^v double-float values per lane over the lanes of a warp and
-// scatters the totals (a reduce-scatter butterfly): at each of the first v
-// levels (lane offsets 16, 8, ...) a lane keeps the half of its values that its
-// lane bit selects and adds the partner's copy of that half; the offsets left,
-// down to OMIN, sum the one value kept. On return (OMIN = 1) lane L holds the
-// total of value L / (32 / V), every lane of a group of 32 / V the same; with
-// OMIN > 1 lanes that differ below OMIN keep separate sums. For V = 32 this is
-// 31 double-float additions per lane on the float32 pipes, where a float64
-// butterfly per value takes 5 V float64 additions: GB300 issues float64 at
-// 1/64 of the float32 rate, and that once-per-tile reduction used to bound the
-// float32 evolution kernel.
-template <int V, int OMIN = 1>
-__device__ __forceinline__ df32 warp_reduce_scatter(df32 (&x)[V], const int lane) {
-    static_assert((V & (V - 1)) == 0 && V <= 32 / OMIN, "V a power of two, at most the lanes summed over");
-#pragma unroll
-    for (int half = V / 2, o = 16; half >= 1; half >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < half; ++i) {
-            const df32 send = up ? x[i] : x[i + half];
-            const df32 keep = up ? x[i + half] : x[i];
-            x[i] = keep + shfl_xor_df(send, o);
-        }
-    }
-    df32 v = x[0];
-#pragma unroll
-    for (int o = 16 / V; o >= OMIN; o >>= 1) v = v + shfl_xor_df(v, o);
     return v;
 }
 
@@ -1014,47 +981,6 @@ reduce_df4:
 // subtraction without a product. Tiles of TB bits in every realization, no
 // two-body flips (those handles launch tile_step_df4 with TB = 0).
 
-// The 16 bytes of a column pair are (hi_p, hi_{p+1} | lo_p, lo_{p+1}): the two
-// register pairs of a DF2 as they are.
-__device__ __forceinline__ DF2 ld_df2_s(const df32* p) {
-    const ulonglong2 f = *reinterpret_cast<const ulonglong2*>(p);
-    return DF2{f.x, f.y};
-}
-
-template <bool COHERENT>
-__device__ __forceinline__ DF2 ld_df2_g(const df32* p) {
-    const ulonglong2 f = COHERENT ? __ldcg(reinterpret_cast<const ulonglong2*>(p))
-                                  : __ldg(reinterpret_cast<const ulonglong2*>(p));
-    return DF2{f.x, f.y};
-}
-
-template <bool COHERENT>
-__device__ __forceinline__ DF2 ld_df2_rw(const df32* p) {
-    const ulonglong2 f = COHERENT ? __ldcg(reinterpret_cast<const ulonglong2*>(p))
-                                  : *reinterpret_cast<const ulonglong2*>(p);
-    return DF2{f.x, f.y};
-}
-
-__device__ __forceinline__ void st_df2(df32* p, DF2 v) {
-    *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v.hi, v.lo);
-}
-
-// lanes swapped: (x1 | x0)
-__device__ __forceinline__ DF2 df2_swap(DF2 v) {
-    float h0, h1, l0, l1;
-    upk2(v.hi, h0, h1);
-    upk2(v.lo, l0, l1);
-    return DF2{pk2(h1, h0), pk2(l1, l0)};
-}
-
-__device__ __forceinline__ DF2 df2_shfl_xor(DF2 v, int o) {
-    float h0, h1, l0, l1;
-    upk2(v.hi, h0, h1);
-    upk2(v.lo, l0, l1);
-    return DF2{pk2(__shfl_xor_sync(0xffffffffu, h0, o), __shfl_xor_sync(0xffffffffu, h1, o)),
-               pk2(__shfl_xor_sync(0xffffffffu, l0, o), __shfl_xor_sync(0xffffffffu, l1, o))};
-}
-
 template <int MODE, bool COHERENT, int TB>
 __device__ __forceinline__ void tile_step_df4x2(const StepArgs& a, const int item, const int step) {
     static_assert(TB > 0, "the paired pass is specialised on the tile's bit count");
@@ -1077,9 +1003,10 @@ __device__ __forceinline__ void tile_step_df4x2(const StepArgs& a, const int ite
     if (MODE != kApply && a.nsteps_override > 0) nsteps = a.nsteps_override;
     const bool active = step < nsteps;
     constexpr bool want_mom = MODE == kEvolve;
-    Dot2x2 mp[5];
+    Dot2x2 mwi[3], mac[2];           // moment sums within the thread's column pair and across the pairs
 #pragma unroll
-    for (int e = 0; e < 5; ++e) mp[e] = Dot2x2{0ull, 0ull};
+    for (int e = 0; e < 3; ++e) mwi[e] = Dot2x2{0ull, 0ull};
+    mac[0] = mac[1] = Dot2x2{0ull, 0ull};
 
     if (active) {
         T* wA = static_cast<T*>(a.bufA);
@@ -1224,24 +1151,8 @@ __device__ __forceinline__ void tile_step_df4x2(const StepArgs& a, const int ite
             if (want_mom) {
                 const DF2 Cx = df2_shfl_xor(A, 1);        // the other pair's x
                 if (val) {
-                    // h = 0: (x0 x0 | x1 x1), (o0 x0 | o1 x1), (x0 x1 | o0 x1), (o0 x2 | o1 x3), (o0 x3 | o1 x2)
-                    // h = 1: the same with columns 2, 3 for 0, 1, and <x_p, x_q> across the pairs
-                    const DF2m Am = df2m(A);
-                    dot2x2_mad(mp[0], Am, A);
-                    dot2x2_mad(mp[1], Am, O);
-                    {
-                        float ah0, ah1, al0, al1, oh0, oh1, ol0, ol1;
-                        upk2(A.hi, ah0, ah1);
-                        upk2(A.lo, al0, al1);
-                        upk2(O.hi, oh0, oh1);
-                        upk2(O.lo, ol0, ol1);
-                        const DF2 X01 = DF2{pk2(ah0, oh0), pk2(al0, ol0)};
-                        dot2x2_mad(mp[2], df2m(X01), DF2{pk2(ah1, ah1), pk2(al1, al1)});
-                    }
-                    const DF2 U = h ? Cx : O, V = h ? A : Cx;
-                    const DF2m Um = df2m(U);
-                    dot2x2_mad(mp[3], Um, V);
-                    dot2x2_mad(mp[4], Um, df2_swap(V));
+                    df4_moments_within(mwi, A, O);
+                    df4_moments_across(mac, A, O, Cx, h);
                 }
             }
         }
@@ -1251,35 +1162,12 @@ __device__ __forceinline__ void tile_step_df4x2(const StepArgs& a, const int ite
 reduce_df4x2:
     if (want_mom && active) {
         const int lane = tid & 31, warp = tid >> 5;
-        // the ten sums in the order of tile_step_df4: (x0x0, x0x1, x1x1, o0x0, o0x1, o1x1,
-        // u0v0, u0v1, u1v0, u1v1) for h = 0; columns shifted by two for h = 1
-        Dot2 ms[10];
-        dot2x2_split(mp[0], ms[0], ms[2]);
-        dot2x2_split(mp[1], ms[3], ms[5]);
-        dot2x2_split(mp[2], ms[1], ms[4]);
-        dot2x2_split(mp[3], ms[6], ms[9]);
-        dot2x2_split(mp[4], ms[7], ms[8]);
-        df32 xs[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) xs[e] = e < 10 ? dot2_final(ms[e]) : df32(0.f, 0.f);
-        const df32 t = warp_reduce_scatter<16, 2>(xs, lane);
-        const int e = (lane >> 1) & 15;
+        int e;
+        const df32 t = df4_warp_moments(mwi, mac, lane, e);
         if (e < 10) {
-            int blk, p, q;
-            if (e < 6) {
-                blk = e / 3;
-                const int k = e % 3;
-                p = 2 * h + (k == 2 ? 1 : 0);
-                q = 2 * h + (k >= 1 ? 1 : 0);
-            } else {
-                blk = h == 0 ? 1 : 0;
-                p = (e - 6) >> 1;
-                q = 2 + ((e - 6) & 1);
-            }
-            const double v = static_cast<double>(t);
-            double* rw = red_s[warp];
-            rw[blk * B * B + p * B + q] = v;
-            rw[blk * B * B + q * B + p] = v;
+            const int2 pq = df4_moment_entry(e, h);
+            red_s[warp][pq.x] = static_cast<double>(t);
+            red_s[warp][pq.y] = static_cast<double>(t);
         }
         __syncthreads();
         if (tid < 2 * B * B) {
@@ -1450,7 +1338,7 @@ static cudaError_t launch_one(const StepArgs& a, int item_base, int n_items, int
 static std::mutex g_smem_mu;
 static std::map<std::pair<const void*, int>, int> g_smem_max;
 
-static cudaError_t grow_smem_attr(const void* func, int smem) {
+cudaError_t grow_smem_attr(const void* func, int smem) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;

@@ -50,7 +50,7 @@ def _flip(m, c):
     return dict(m, gflip=c)
 
 
-PRECS = [("fp64", P.DACP_FP64, 2.0 ** -53)]
+PRECS = [("fp64", P.DACP_FP64, 2.0 ** -53), ("df32", P.DACP_DF32, 2.0 ** -44)]
 
 
 @pytest.mark.parametrize("name,prec,unit", PRECS)
@@ -84,6 +84,31 @@ def test_start_vectors_of_one_state_and_of_uneven_size(N, name, prec, unit):
     decay[::2, 1] *= 0.5
     models = [W.random_model(N, seed=80 + i) for i in range(3)]
     _check(models, [one, W.start_vectors(N, 2, seed=6), decay], 2, 30, prec, unit)
+
+
+@pytest.mark.parametrize("flip", [False, True])
+@pytest.mark.parametrize("N,tile", [(13, 32768), (14, 65536)])
+def test_double_float_clusters_keep_the_bits_of_the_per_order_launch(N, tile, flip):
+    """16 realizations of 8 tiles take the per-order launch, the first two of them alone a cluster each: their
+    moments equal to the last bit."""
+    models = [W.spin_glass_shard(N, seed=20 + r) for r in range(16)]
+    if flip:
+        models = [_flip(m, 0.7 - 0.01 * r) for r, m in enumerate(models)]
+    psis = [W.start_vectors(N, 4, seed=8, r=r) for r in range(16)]
+    emax = np.array([_bound(m) for m in models])
+    mu = []
+    for count in (16, 2):
+        d = P.Dacp(models[:count], psis[:count], block_b=4, precision=P.DACP_DF32)
+        try:
+            d.set_launch(0, tile)
+            d.set_params(emax[:count], 0.1 * emax[:count], 5, 2 + np.arange(count) % 2)
+            d.filter()
+            d.basis_moments()
+            mu.append([d.moments(r) for r in range(2)])
+        finally:
+            d.close()
+    for a, b in zip(*mu):
+        assert np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("name,prec,unit", PRECS)
