@@ -71,11 +71,20 @@ struct FxMom {
         mm += static_cast<int64_t>(ah) * bl;
         mm += static_cast<int64_t>(al) * bh;
     }
-    // in units of 2^(58 + shift); half: 2^(shift - 1), one less on every other thread so that the halves do not add up
-    __device__ __forceinline__ int64_t fold(int shift, int half) const {
-        return (hh + ((mm + (int64_t(1) << 28)) >> 29) + half) >> shift;
-    }
+    // the sum in units of 2^58
+    __device__ __forceinline__ int64_t value() const { return hh + ((mm + (int64_t(1) << 28)) >> 29); }
 };
+
+// A sum of moment products over lanes: hi 2^8 + lo, so that no vector can overflow it.
+struct FxSum {
+    int64_t hi;
+    int lo;
+};
+__device__ __forceinline__ FxSum operator+(const FxSum a, const FxSum b) { return FxSum{a.hi + b.hi, a.lo + b.lo}; }
+__device__ __forceinline__ FxSum warp_shfl_xor(const FxSum v, int o) {
+    return FxSum{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ FxSum fx_sum(const int64_t v) { return FxSum{v >> 8, static_cast<int>(v & 255)}; }
 
 // Barrier of the realization's group: the CTA alone, a cluster, or CTAs of a cooperative launch
 // on a counter (bounded: false when one second passes, and then at every CTA of the group).
@@ -137,7 +146,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     constexpr int LU = U == 4 ? 2 : (U == 2 ? 1 : 0);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int2 g_s[kMaxSpins + 1];            // 2 Gamma_i / E_max, then the global flip
-    __shared__ long long red_s[kFxRedRing][kFxThreads / 32][NS];
+    __shared__ FxSum red_s[kFxRedRing][kFxThreads / 32][NS];
     __shared__ float pro_s[3][kFxThreads / 32];
     __shared__ float max_s[4];
 
@@ -238,12 +247,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     // coefficients in units of 2^-(58 - ge): as fine as the sum of their magnitudes allows (limbs and 64-bit sums)
     const int ge = gsum < 3.95 ? 0 : 1;
     const double cg = ldexp(c2, 58 - ge);
-    // A warp's sum of products stays below 2^62 after a shift by msh: it is at most the squared norm
-    // (Cauchy-Schwarz) and at most its T / nwarps products of 2^58 each, in units of 2^58.
-    const int norm2 = ilogbf(ss) + 1 + 2 * sexp - 58 - 61;
-    const int most = 32 - __clz(T / nwarps) - 3;
-    const int msh = max(0, min(norm2, most));
-    const int half = msh > 0 ? (1 << (msh - 1)) - (tid & 1) : 0;
     if (tid < R.N) g_s[tid] = fx_limbs(__double2ll_rn(cg * a.gam[r * kMaxSpins + tid]));
     if (tid == kMaxSpins) g_s[kMaxSpins] = a.gflip ? fx_limbs(__double2ll_rn(cg * a.gflip[r])) : make_int2(0, 0);
     const int64_t pslot0 = R.off * B / 2;           // the realization's first published slot (off is a multiple of 4)
@@ -262,7 +265,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     }
     if (!fx_group_sync(a, group, target += G, [] {})) return;
 
-    const double unit = ldexp(1.0, 58 + msh - 2 * sexp);
+    const double unit = ldexp(1.0, 58 - 2 * sexp);
     const double square = ldexp(1.0 / 3.0, R.N + 56 - 2 * sexp);
     longlong2* part = a.part + static_cast<int64_t>(group) * kFxPartRing * NS;
     const int64_t row0 = a.mom_rows_fixed > 0 ? static_cast<int64_t>(r) * a.mom_rows_fixed : R.mom_off;
@@ -308,9 +311,9 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
         if (active && lane < NS && k >= 1 && k <= orders) {
             long long hi = 0, lo = 0;
             for (int w = 0; w < nwarps; ++w) {
-                const long long s = red_s[(k - 1) % kFxRedRing][w][lane];
-                hi += s >> 24;
-                lo += s & ((1 << 24) - 1);
+                const FxSum s = red_s[(k - 1) % kFxRedRing][w][lane];
+                hi += s.hi >> 16;
+                lo += (s.hi & 0xffff) * 256 + s.lo;
             }
             // integer sums: the order in which the CTAs add does not matter
             unsigned long long* slot = reinterpret_cast<unsigned long long*>(part + ((k - 1) % kFxPartRing) * NS + lane);
@@ -472,21 +475,21 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
             }
             // the warp's sums, lane by lane
             if constexpr (B == 4) {
-                int64_t v[16];
+                FxSum v[16];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) v[e] = e < 10 ? ms[e].fold(msh, half) : 0;
-                const int64_t s = warp_reduce_scatter<16, 2>(v, lane);
+                for (int e = 0; e < 16; ++e) v[e] = fx_sum(e < 10 ? ms[e].value() : 0);
+                const FxSum s = warp_reduce_scatter<16, 2>(v, lane);
                 const int e = lane >> 1;
                 if (e < 10) red_s[k % kFxRedRing][warp][(lane & 1) * 10 + e] = s;
             } else if constexpr (B == 2) {
-                int64_t v[8];
+                FxSum v[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = e < 6 ? ms[e].fold(msh, half) : 0;
-                const int64_t s = warp_reduce_scatter<8>(v, lane);
+                for (int e = 0; e < 8; ++e) v[e] = fx_sum(e < 6 ? ms[e].value() : 0);
+                const FxSum s = warp_reduce_scatter<8>(v, lane);
                 if ((lane & 3) == 0 && (lane >> 2) < 6) red_s[k % kFxRedRing][warp][lane >> 2] = s;
             } else {
-                int64_t v[2] = {ms[0].fold(msh, half), ms[1].fold(msh, half)};
-                const int64_t s = warp_reduce_scatter<2>(v, lane);
+                FxSum v[2] = {fx_sum(ms[0].value()), fx_sum(ms[1].value())};
+                const FxSum s = warp_reduce_scatter<2>(v, lane);
                 if ((lane & 15) == 0) red_s[k % kFxRedRing][warp][lane >> 4] = s;
             }
         }
@@ -523,7 +526,7 @@ const void* fx_kernel_b(int u) {
 
 const void* fx_kernel(int b, int u) { return b == 4 ? fx_kernel_b<4>(u) : (b == 2 ? fx_kernel_b<2>(u) : fx_kernel_b<1>(u)); }
 
-constexpr int kFxStatic = 10240;        // static shared memory of the kernels, rounded up
+constexpr int kFxStatic = 18432;        // static shared memory of the kernels, rounded up
 
 int fx_smem(int b, int maxN, int lg) {
     const int64_t T = int64_t(1) << (maxN - lg > 0 ? maxN - lg : 0);

@@ -10,9 +10,8 @@ __device__ __forceinline__ df32 shfl_xor_df(df32 v, int o) {
 }
 
 __device__ __forceinline__ df32 warp_shfl_xor(df32 v, int o) { return shfl_xor_df(v, o); }
-__device__ __forceinline__ int64_t warp_shfl_xor(int64_t v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 
-// Sums V = 2^v double-float values (or 64-bit integers) per lane over the lanes of a warp and
+// Sums V = 2^v values (double-float, or any type with + and warp_shfl_xor) per lane over the lanes of a warp and
 // scatters the totals (a reduce-scatter butterfly): at each of the first v
 // levels (lane offsets 16, 8, ...) a lane keeps the half of its values that its
 // lane bit selects and adds the partner's copy of that half; the offsets left,
