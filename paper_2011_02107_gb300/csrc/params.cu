@@ -159,7 +159,7 @@ __device__ __forceinline__ double warp_max_d(double v) {
     return v;
 }
 
-constexpr int kBoundWarps = 4;
+constexpr int kBoundWarps = 1;   // one warp a block: the bisections are float64 divisions, which warps of an SM share
 
 // Extreme Ritz values by bisection; bound = max(|theta_min|, |theta_max|) + beta_{k+1}
 // (rule 0) or the Ritz-residual rule (rule 1), times (1 + safety), clamped to the
@@ -211,14 +211,20 @@ __global__ void __launch_bounds__(32 * kBoundWarps) lanczos_bound_kernel(int R, 
 // in [-a_r, a_r] = D [g_0 mu_0 (pi - 2 phi)/pi + 2 sum g_j mu_j (sin(j(pi-phi)) - sin(j phi))/(pi j)],
 // phi = acos(a_r); bisection for count = d_target. Then K = ceil(c E_max / a)
 // and n = ceil((basis_ratio d / b - 1) / 2).
-__global__ void kpm_window_kernel(int R, const RealInfo* __restrict__ real, const double* __restrict__ P,
+constexpr int kWindowTerms = 2048;    // terms kept in shared memory (the default takes 256)
+
+__global__ void __launch_bounds__(32) kpm_window_kernel(int R, const RealInfo* __restrict__ real, const double* __restrict__ P,
                                   int M, const double* __restrict__ emax, double d_target, double c_order,
                                   double basis_ratio, int b, const float* __restrict__ knobs, int n_eigs,
                                   double* a_out, int* K_out, int* n_out) {
-    // one warp per realization: the lanes share the moment sum of each count evaluation
-    const int r = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x & 31;
-    if (r >= R) return;
+    // One warp per realization and block: the lanes share the moment sum of each count evaluation, whose two
+    // sines a term are what the search takes its time for (float64 at 1.7 operations per clock and SM), so
+    // no second warp shares the SM while there are SMs left, and the factors that do not depend on the
+    // candidate stay in shared memory. (Four warps a block, every factor evaluated anew and 100 halvings
+    // took most of the parameter choice.)
+    const int r = blockIdx.x;
+    const int lane = threadIdx.x;
+    __shared__ double term_s[kWindowTerms];
     if (knobs) {
         // learned knobs per realization: log(window ratio), filter constant, basis ratio;
         // clamped to the range the network was trained on
@@ -230,13 +236,18 @@ __global__ void kpm_window_kernel(int R, const RealInfo* __restrict__ real, cons
     const double* Pr = P + static_cast<int64_t>(r) * M;
     const double q = M_PI / (M + 1);
     const double cq = 1.0 / tan(q);
+    auto term = [&](int j) {
+        const double g = ((M - j + 1) * cos(q * j) + sin(q * j) * cq) / (M + 1);
+        const double mu = 2.0 * Pr[j] - Pr[j & 1];
+        return 2.0 * g * mu;
+    };
+    for (int j = 1 + lane; j < M && j < kWindowTerms; j += 32) term_s[j] = term(j);    // read by the same lane
     auto count = [&](double ar) {
         const double phi = acos(ar);
         double tot = lane == 0 ? Pr[0] * (M_PI - 2.0 * phi) / M_PI : 0.0;   // g_0 = 1, mu_0 = P_0
         for (int j = 1 + lane; j < M; j += 32) {
-            const double g = ((M - j + 1) * cos(q * j) + sin(q * j) * cq) / (M + 1);
-            const double mu = 2.0 * Pr[j] - Pr[j & 1];
-            tot += 2.0 * g * mu * (sin(j * (M_PI - phi)) - sin(j * phi)) / (M_PI * j);
+            const double t = j < kWindowTerms ? term_s[j] : term(j);
+            tot += t * (sin(j * (M_PI - phi)) - sin(j * phi)) / (M_PI * j);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
@@ -250,6 +261,7 @@ __global__ void kpm_window_kernel(int R, const RealInfo* __restrict__ real, cons
         double lo = 0.0, hi = 0.999;
         for (int it = 0; it < 100; ++it) {
             const double mid = 0.5 * (lo + hi);
+            if (mid == lo || mid == hi) break;     // neighbours: further halvings change neither
             if (count(mid) < d_target) lo = mid; else hi = mid;
         }
         a = 0.5 * (lo + hi) * em;
@@ -302,7 +314,7 @@ cudaError_t launch_lanczos_bound(int R, const double* lmom, int rows, const doub
 cudaError_t launch_kpm_window(int R, const RealInfo* real, const double* P, int M, const double* emax,
                               double d_target, double c_order, double basis_ratio, int b, const float* knobs,
                               int n_eigs, double* a_out, int* K_out, int* n_out, cudaStream_t st) {
-    kpm_window_kernel<<<(R + 3) / 4, 128, 0, st>>>(R, real, P, M, emax, d_target, c_order, basis_ratio, b, knobs,
+    kpm_window_kernel<<<R, 32, 0, st>>>(R, real, P, M, emax, d_target, c_order, basis_ratio, b, knobs,
                                                    n_eigs, a_out, K_out, n_out);
     return cudaGetLastError();
 }
