@@ -645,15 +645,48 @@ dacp_status fx_finish(dacp_ctx* c, const FxRun& q, const std::vector<double>& em
     return DACP_OK;
 }
 
-// Whether the evolution of launch mode 0 runs as resident double-float clusters, one CTA per tile of the
-// per-order launch (whose bits it keeps). Clusters of up to 4 CTAs win at every batch size: 4.11 against 8.00 ms
-// for 361 orders of 36 13-spin sectors, 61.4 against 64.8 ms of 512. Of 8 CTAs only 15 fit the GPU (120 of
-// 152 SMs), so there the per-order launch is ahead once they do not all run at once: 79.1 against 65.2 ms
-// for 256 14-spin shards.
+// Whether the recurrences of launch mode 0 run as resident double-float clusters, one CTA per tile of the
+// per-order launch (whose bits they keep). Clusters of up to 4 CTAs win at every batch size: 4.11 against
+// 8.00 ms for 361 evolution orders of 36 13-spin sectors, 61.4 against 64.8 ms of 512. Of 8 CTAs only 15 fit
+// the GPU (120 of 152 SMs), so there the per-order launch is ahead once they do not all run at once: 79.1
+// against 65.2 ms for 256 14-spin shards.
 bool df_resident_usable(const dacp_ctx* c) {
     if (c->prec != kPrecDF32 || c->b != 4 || c->has_pairs || c->launch_mode != 0) return false;
     const int max_N = *std::max_element(c->N.begin(), c->N.end());
     return df4_resident_fits(c->tb_uniform, max_N) && (max_N - c->tb_uniform < 3 || c->R <= 15);
+}
+
+DfResArgs df_resident_args(const dacp_ctx* c) {
+    DfResArgs a;
+    memset(&a, 0, sizeof(a));
+    while (c->tb_uniform + a.lg < *std::max_element(c->N.begin(), c->N.end())) ++a.lg;
+    a.real = c->info_d;
+    a.diag = static_cast<const df32*>(c->diag_d);
+    a.gam = static_cast<const df32*>(c->gam_d);
+    a.gflip = c->has_gflip ? c->gflip_d : nullptr;
+    a.emax = c->fx_emax_d;
+    a.coef = c->coef_d;
+    a.psi = c->psiE_d;
+    a.pub0 = static_cast<ulonglong2*>(c->A_d);
+    a.pub1 = static_cast<ulonglong2*>(c->B_d);
+    a.pubu = static_cast<ulonglong2*>(c->U_d);
+    a.part = c->df_part_d;
+    a.mom = c->mom_d;
+    return a;
+}
+
+// Queue the filter's recurrence of every realization, w_0 in A, longest run first.
+dacp_status df_resident_filter(dacp_ctx* c) {
+    TRY(resident_lists(c));
+    std::vector<int> list(c->R);
+    std::iota(list.begin(), list.end(), 0);
+    std::stable_sort(list.begin(), list.end(), [&](int x, int y) { return c->K[x] > c->K[y]; });
+    CK(cudaMemcpyAsync(c->fx_list_d, list.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
+    DfResArgs a = df_resident_args(c);
+    a.list = c->fx_list_d;
+    CK(launch_df4_resident(c->tb_uniform, true, a, c->R, c->st));
+    c->launches += 1;
+    return DACP_OK;
 }
 
 // Queue the resident double-float evolution of the realizations order[0 .. R), group by group: group g is
@@ -663,9 +696,7 @@ bool df_resident_usable(const dacp_ctx* c) {
 dacp_status df_resident_launch(dacp_ctx* c, const std::vector<int>& order, const std::vector<int>& from,
                                const std::vector<cudaStream_t>& st) {
     TRY(resident_lists(c));
-    DfResArgs a;
-    memset(&a, 0, sizeof(a));
-    for (a.lg = 0; c->tb_uniform + a.lg < *std::max_element(c->N.begin(), c->N.end());) ++a.lg;
+    DfResArgs a = df_resident_args(c);
     const size_t parts = (static_cast<size_t>(c->R) << a.lg) * kDfPartSums;
     if (parts > c->df_parts) {
         dfree(c, c->df_part_d);
@@ -682,20 +713,11 @@ dacp_status df_resident_launch(dacp_ctx* c, const std::vector<int>& order, const
     CK(cudaMemcpyAsync(c->fx_emax_d, c->emax.data(), sizeof(double) * c->R, cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(c->fx_list_d, list.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
     CK(cudaEventRecord(c->ev[2], c->st));            // also the start of T_E
-    a.real = c->info_d;
-    a.diag = static_cast<const df32*>(c->diag_d);
-    a.gam = static_cast<const df32*>(c->gam_d);
-    a.gflip = c->has_gflip ? c->gflip_d : nullptr;
-    a.emax = c->fx_emax_d;
-    a.psi = c->psiE_d;
-    a.pub0 = static_cast<ulonglong2*>(c->A_d);
-    a.pub1 = static_cast<ulonglong2*>(c->B_d);
-    a.mom = c->mom_d;
     for (int g = 0; g < ng; ++g) {
         if (st[g] != c->st) CK(cudaStreamWaitEvent(st[g], c->ev[2], 0));
         a.list = c->fx_list_d + from[g];
         a.part = c->df_part_d + (static_cast<size_t>(from[g]) << a.lg) * kDfPartSums;
-        CK(launch_evolve_df4_resident(c->tb_uniform, a, from[g + 1] - from[g], st[g]));
+        CK(launch_df4_resident(c->tb_uniform, false, a, from[g + 1] - from[g], st[g]));
         c->launches += 1;
     }
     return DACP_OK;
@@ -1182,7 +1204,8 @@ dacp_status dacp_filter(dacp_handle c) {
     for (int r = 0; r < c->R; ++r) maxK = std::max(maxK, c->K[r]);
     CK(cudaEventRecord(c->ev[0], c->st));
     CK(cudaMemcpyAsync(c->A_d, c->psi0_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
-    TRY(run_orders(c, true, maxK));
+    if (df_resident_usable(c)) TRY(df_resident_filter(c));
+    else TRY(run_orders(c, true, maxK));
     // psi_E = w_K / |w_K| per column; w_K sits in A (K even) or B (K odd); also w_0 of the evolution
     c->launches += 2;
     CK(launch_normalize(c->prec, c->b, c->items_d, c->info_d, static_cast<int>(c->items.size()), c->A_d, c->B_d, 1,

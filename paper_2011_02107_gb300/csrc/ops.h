@@ -61,21 +61,23 @@ int fx_part_sums(int b);            // elements of FxArgs::part per group
 bool fx_plan(int b, int count, int minN, int maxN, FxPlan* p);
 cudaError_t launch_evolve_fx(int b, const FxPlan& p, const FxArgs& a, int count, cudaStream_t st);
 
-// resident_df.cu: the double-float b = 4 evolution with both vectors in shared memory
+// resident_df.cu: the double-float b = 4 recurrences with their vectors in shared memory
 struct DfResArgs {
     const int* list;                // realizations, one cluster of 2^lg CTAs each
     const RealInfo* real;
     const df32 *diag, *gam;
-    const double *gflip, *emax;     // [R]; gflip nullptr: none
-    const void* psi;
-    ulonglong2 *pub0, *pub1;        // published vectors, as a vector of the batch
+    const double* gflip;            // [R]; nullptr: none
+    const double* emax;             // [R] (evolution)
+    const double* coef;             // [R][8] (filter)
+    const void* psi;                // w_0 of the evolution
+    ulonglong2 *pub0, *pub1, *pubu;  // published w_k (even, odd k) and u = H w_k, as vectors of the batch
     double* part;                   // [clusters][4][2^lg][32] moment sums in flight
     double* mom;
     int lg;
 };
 constexpr int kDfPartSums = 4 * 32; // doubles of DfResArgs::part per CTA
 bool df4_resident_fits(int tbits_uniform, int max_N);
-cudaError_t launch_evolve_df4_resident(int tbits, const DfResArgs& a, int count, cudaStream_t st);
+cudaError_t launch_df4_resident(int tbits, bool filter, const DfResArgs& a, int count, cudaStream_t st);
 
 // subspace.cu
 cudaError_t launch_orders(int L, double a_r, int* orders, cudaStream_t st);

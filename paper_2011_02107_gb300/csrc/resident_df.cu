@@ -1,9 +1,9 @@
-// The double-float b = 4 evolution w_{k+1} = 2 G w_k - w_{k-1} (Sec. II B) with
-// both vectors of a realization resident in shared memory for the whole run.
+// The double-float b = 4 recurrences, filter (Sec. II A) and evolution (Sec. II B), with
+// the vectors of a realization resident in shared memory for the whole run.
 //
 // A cluster owns one realization, one CTA per tile of the per-order launch
 // (2^(N - TB) tiles of 2^TB states). Its tiles of w_k and w_{k-1} (overwritten
-// by w_{k+1}) and its diagonal stay in shared memory from the first order to
+// by w_{k+1}; the filter also of u = H w_k) and its diagonal stay in shared memory from the first order to
 // the last, and one cluster barrier (0.23 us) separates the orders. A flip of
 // a bit beyond the tile, and the global flip, reads the partner CTA's tile:
 // each CTA also publishes its new tile to global memory, where it stays in L2
@@ -28,6 +28,94 @@ namespace {
 constexpr int kDfThreads = 2 * kThreads;
 constexpr int kRedRing = 3, kPartRing = 4;          // orders in flight between a sum and its moment row
 constexpr int kRowSums = 32;                        // two rows of 4 x 4
+
+// Scaled x-fields in shared memory, per spin (g.hi, g.hi, g.lo, g.lo) and (-g.hi, -g.hi): the register
+// pairs of a DF2m. Entry kMaxSpins is the global flip.
+struct Df4Fields {
+    const ulonglong2* g;
+    const uint64_t* ng;
+    __device__ __forceinline__ DF2m operator[](const int i) const { return DF2m{g[i].x, ng[i], g[i].y}; }
+};
+
+__device__ __forceinline__ void df4_load_fields(float4* g_s, float2* ng_s, const df32 ch, const df32* gam,
+                                                const double* gflip, const int N) {
+    const int i = threadIdx.x;
+    if (i < N || (i == kMaxSpins && gflip)) {
+        const df32 g = ch * (i < N ? gam[i] : df32(*gflip));
+        g_s[i] = make_float4(g.hi, g.hi, g.lo, g.lo);
+        ng_s[i] = make_float2(-g.hi, -g.hi);
+    }
+}
+
+// The flips of U slots (base, base + kDfThreads, ...) of the tile `cur`, in rising bit order, then the global
+// flip; A: the slots themselves. pcur: the realization's published vector.
+template <int TB, int U>
+__device__ __forceinline__ void df4_flips(const ulonglong2* cur, const ulonglong2* pcur, const int base, const int rank,
+                                          const int nb, const bool gflip, const Df4Fields gam, DF2 (&A)[U],
+                                          Dot2x2 (&acc)[U]) {
+    constexpr int kSlots = 2 << TB;
+    auto at = [&](const int sl) {
+        const ulonglong2 v = cur[sl];
+        return DF2{v.x, v.y};
+    };
+    DF2 P[3][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) A[u] = at(base + kDfThreads * u);
+    // partner tiles: loaded now, summed after the flips inside the tile
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const bool flip = j >= nb;                   // the first slot past the bits: the global flip
+        if (j < nb || (j == nb && gflip && nb > 0)) {
+            const ulonglong2* pp = pcur + (flip ? rank ^ ((1 << nb) - 1) : rank ^ (1 << j)) * kSlots;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int sl = base + kDfThreads * u;
+                const ulonglong2 v = __ldcg(pp + (flip ? sl ^ (kSlots - 2) : sl));
+                P[j][u] = DF2{v.x, v.y};
+            }
+        }
+    }
+    {
+        const DF2m g = gam[0];
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc[u] = dot2x2_prod(g, at((base + kDfThreads * u) ^ 2));
+    }
+#pragma unroll
+    for (int i = 1; i < TB; ++i) {
+        const DF2m g = gam[i];
+        // the bit's distance in slots; two of them lie among the thread's own slots
+        const int dist = 2 << i, du = dist / kDfThreads;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            dot2x2_mad(acc[u], g, du >= 1 && du < U ? A[u ^ du] : at((base + kDfThreads * u) ^ dist));
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        if (j < nb || (j == nb && gflip && nb > 0)) {
+            const DF2m g = gam[j < nb ? TB + j : kMaxSpins];
+#pragma unroll
+            for (int u = 0; u < U; ++u) dot2x2_mad(acc[u], g, P[j][u]);
+        }
+    }
+    if (gflip && (nb == 0 || nb == 3)) {             // one tile, or no early slot left
+        const DF2m g = gam[kMaxSpins];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int sl = (base + kDfThreads * u) ^ (kSlots - 2);
+            const ulonglong2 v = nb == 0 ? cur[sl] : __ldcg(pcur + (rank ^ ((1 << nb) - 1)) * kSlots + sl);
+            dot2x2_mad(acc[u], g, DF2{v.x, v.y});
+        }
+    }
+}
+
+__device__ __forceinline__ void df4_cluster_sync(const bool cluster) {
+    if (cluster) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+        __syncthreads();
+    }
+}
 
 // Bound by the float32 pipe (248 lane operations per value and order at 13 spins and a global flip).
 // Two passes an order, so that 16 warps of an SM work although the moments have 256 running sums of
@@ -59,22 +147,12 @@ __global__ void __launch_bounds__(kDfThreads, 1) evolve_df4_resident_kernel(cons
     ulonglong2* buf1 = buf0 + kSlots;
     df32* diag_s = reinterpret_cast<df32*>(buf1 + kSlots);
     const int64_t slot0 = R.off * 2 + static_cast<int64_t>(rank) * kSlots;
-    const ulonglong2* g2 = reinterpret_cast<const ulonglong2*>(gam_s);
-    const uint64_t* ng2 = reinterpret_cast<const uint64_t*>(ngam_s);
+    const Df4Fields gam{reinterpret_cast<const ulonglong2*>(gam_s), reinterpret_cast<const uint64_t*>(ngam_s)};
     const bool gflip = a.gflip != nullptr;
     // 2 / E_max in every order: order 0 (w_1 = G w_0) takes half of its sum, which is exact
     const df32 ch = static_cast<df32>(2.0 / a.emax[r]);
 
-    if (tid < R.N) {
-        const df32 g = ch * a.gam[r * kMaxSpins + tid];
-        gam_s[tid] = make_float4(g.hi, g.hi, g.lo, g.lo);
-        ngam_s[tid] = make_float2(-g.hi, -g.hi);
-    }
-    if (tid == kMaxSpins && gflip) {
-        const df32 g = ch * df32(a.gflip[r]);
-        gam_s[kMaxSpins] = make_float4(g.hi, g.hi, g.lo, g.lo);
-        ngam_s[kMaxSpins] = make_float2(-g.hi, -g.hi);
-    }
+    df4_load_fields(gam_s, ngam_s, ch, a.gam + r * kMaxSpins, gflip ? a.gflip + r : nullptr, R.N);
     if (active) {
         const ulonglong2* psi = static_cast<const ulonglong2*>(a.psi) + slot0;
         for (int i = tid; i < kSlots; i += kDfThreads) {
@@ -133,60 +211,9 @@ __global__ void __launch_bounds__(kDfThreads, 1) evolve_df4_resident_kernel(cons
         if (active) {
 #pragma unroll 1
             for (int base = tid; base < kSlots; base += kDfThreads * U) {
-                auto at = [&](const int sl) {
-                    const ulonglong2 v = cur[sl];
-                    return DF2{v.x, v.y};
-                };
-                auto coef = [&](const int i) { return DF2m{g2[i].x, ng2[i], g2[i].y}; };
-                DF2 A[U], P[3][U];
+                DF2 A[U];
                 Dot2x2 acc[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) A[u] = at(base + kDfThreads * u);
-                // partner tiles: loaded now, summed after the flips inside the tile
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const bool flip = j >= nb;               // the first slot past the bits: the global flip
-                    if (j < nb || (j == nb && gflip && nb > 0)) {
-                        const ulonglong2* pp = pcur + (flip ? rank ^ ((1 << nb) - 1) : rank ^ (1 << j)) * kSlots;
-#pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            const int sl = base + kDfThreads * u;
-                            const ulonglong2 v = __ldcg(pp + (flip ? sl ^ (kSlots - 2) : sl));
-                            P[j][u] = DF2{v.x, v.y};
-                        }
-                    }
-                }
-                {
-                    const DF2m g = coef(0);
-#pragma unroll
-                    for (int u = 0; u < U; ++u) acc[u] = dot2x2_prod(g, at((base + kDfThreads * u) ^ 2));
-                }
-#pragma unroll
-                for (int i = 1; i < TB; ++i) {
-                    const DF2m g = coef(i);
-                    // the bit's distance in slots; two of them lie among the thread's own slots
-                    const int dist = 2 << i, du = dist / kDfThreads;
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        dot2x2_mad(acc[u], g, du >= 1 && du < U ? A[u ^ du] : at((base + kDfThreads * u) ^ dist));
-                }
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    if (j < nb || (j == nb && gflip && nb > 0)) {
-                        const DF2m g = coef(j < nb ? TB + j : kMaxSpins);
-#pragma unroll
-                        for (int u = 0; u < U; ++u) dot2x2_mad(acc[u], g, P[j][u]);
-                    }
-                }
-                if (gflip && (nb == 0 || nb == 3)) {         // one tile, or no early slot left
-                    const DF2m g = coef(kMaxSpins);
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int sl = (base + kDfThreads * u) ^ (kSlots - 2);
-                        const ulonglong2 v = nb == 0 ? cur[sl] : __ldcg(pcur + (rank ^ ((1 << nb) - 1)) * kSlots + sl);
-                        dot2x2_mad(acc[u], g, DF2{v.x, v.y});
-                    }
-                }
+                df4_flips<TB, U>(cur, pcur, base, rank, nb, gflip, gam, A, acc);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int sl = base + kDfThreads * u;
@@ -245,10 +272,99 @@ __global__ void __launch_bounds__(kDfThreads, 1) evolve_df4_resident_kernel(cons
     for (int k = orders; k < orders + 3; ++k) sync(k);
 }
 
+// The filter's recurrence w_{k+1} = 2 F w_k - w_{k-1}, F = (H^2 - E_c) / E_0 (Sec. II A), with w_k, w_{k-1}
+// (overwritten by w_{k+1}), u = H w_k and the diagonal resident: two passes and two cluster barriers an order.
+// w_K ends in pub0 (K even) or pub1 (K odd), as the per-order launch leaves it. pub0 holds w_0 at the start.
 template <int TB>
-cudaError_t launch_df4_resident(const DfResArgs& a, int count, cudaStream_t st) {
-    auto* f = evolve_df4_resident_kernel<TB>;
-    const int smem = 72 << TB;                      // two vectors of 32 bytes a state and the diagonal
+__global__ void __launch_bounds__(kDfThreads, 1) filter_df4_resident_kernel(const DfResArgs a) {
+    constexpr int kSlots = 2 << TB, NI = kSlots / kDfThreads, U = NI < 4 ? NI : 4;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) float4 gam_s[2][kMaxSpins + 1];     // of u = H w_k, and of w_{k+1}
+    __shared__ __align__(8) float2 ngam_s[2][kMaxSpins + 1];
+
+    const int tid = threadIdx.x;
+    const int group = blockIdx.x >> a.lg, rank = blockIdx.x & ((1 << a.lg) - 1);
+    const int r = a.list[group];
+    const RealInfo R = a.real[r];
+    const int nb = R.N - TB;
+    const bool active = rank < (1 << nb);
+    const int orders = R.nf;
+    ulonglong2* buf0 = reinterpret_cast<ulonglong2*>(smem_raw);
+    ulonglong2* buf1 = buf0 + kSlots;
+    ulonglong2* bufu = buf1 + kSlots;
+    df32* diag_s = reinterpret_cast<df32*>(bufu + kSlots);
+    const int64_t slot0 = R.off * 2 + static_cast<int64_t>(rank) * kSlots;
+    const bool gflip = a.gflip != nullptr;
+    // the coefficients of orders 1, 2, ...; order 0 takes half of their sum without w_{k-1}, which is exact
+    const double* cf = a.coef + 8 * r + 3;
+    const df32 ch = static_cast<df32>(cf[0]);
+    const bool use1 = cf[1] != 0.0, sub1 = cf[1] == -1.0, use2 = cf[2] != 0.0, sub2v = cf[2] == -1.0;
+    const DF2m C1 = df2m_bcast(static_cast<df32>(cf[1])), C2 = df2m_bcast(static_cast<df32>(cf[2]));
+    for (int p = 0; p < 2; ++p)
+        df4_load_fields(gam_s[p], ngam_s[p], p == 0 ? df32(1.0) : ch, a.gam + r * kMaxSpins, gflip ? a.gflip + r : nullptr,
+                        R.N);
+    if (active) {
+        for (int i = tid; i < kSlots; i += kDfThreads) buf0[i] = a.pub0[slot0 + i];
+        for (int i = tid; i < (1 << TB); i += kDfThreads)
+            diag_s[i] = a.diag[R.off + (static_cast<int64_t>(rank) << TB) + i];
+    }
+    df4_cluster_sync(a.lg > 0);
+
+    for (int k = 0; k < orders; ++k) {
+        const ulonglong2* cur = (k & 1) ? buf1 : buf0;
+        ulonglong2* oth = (k & 1) ? buf0 : buf1;
+        const ulonglong2* pcur = ((k & 1) ? a.pub1 : a.pub0) + R.off * 2;
+        ulonglong2* pnew = ((k & 1) ? a.pub0 : a.pub1) + slot0;
+        for (int pass = 0; pass < 2; ++pass) {
+            if (active) {
+                const Df4Fields gam{reinterpret_cast<const ulonglong2*>(gam_s[pass]),
+                                    reinterpret_cast<const uint64_t*>(ngam_s[pass])};
+                const ulonglong2* x = pass == 0 ? cur : bufu;
+                const ulonglong2* px = pass == 0 ? pcur : a.pubu + R.off * 2;
+                ulonglong2* out = pass == 0 ? bufu : oth;
+                ulonglong2* pout = pass == 0 ? a.pubu + slot0 : pnew;
+                const df32 cd = pass == 0 ? df32(1.0) : ch;
+                const bool publish = nb > 0 || (pass == 1 && k == orders - 1);
+#pragma unroll 1
+                for (int base = tid; base < kSlots; base += kDfThreads * U) {
+                    DF2 A[U];
+                    Dot2x2 acc[U];
+                    df4_flips<TB, U>(x, px, base, rank, nb, gflip, gam, A, acc);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int sl = base + kDfThreads * u;
+                        dot2x2_mad(acc[u], df2m_bcast(cd * diag_s[sl >> 1]), A[u]);
+                        if (pass == 1) {
+                            if (use1) {
+                                const ulonglong2 y = cur[sl];
+                                if (sub1) dot2x2_sub(acc[u], DF2{y.x, y.y});
+                                else dot2x2_mad(acc[u], C1, DF2{y.x, y.y});
+                            }
+                            if (use2 && k > 0) {
+                                const ulonglong2 z = oth[sl];
+                                if (sub2v) dot2x2_sub(acc[u], DF2{z.x, z.y});
+                                else dot2x2_mad(acc[u], C2, DF2{z.x, z.y});
+                            }
+                        }
+                        DF2 O = dot2x2_final(acc[u]);
+                        if (pass == 1 && k == 0) {
+                            const uint64_t half = pk2(0.5f, 0.5f);
+                            O = DF2{mul2(O.hi, half), mul2(O.lo, half)};
+                        }
+                        out[sl] = make_ulonglong2(O.hi, O.lo);
+                        if (publish) pout[sl] = make_ulonglong2(O.hi, O.lo);
+                    }
+                }
+            }
+            df4_cluster_sync(a.lg > 0);
+        }
+    }
+}
+
+template <int TB>
+cudaError_t launch_df4_resident(bool filter, const DfResArgs& a, int count, cudaStream_t st) {
+    auto* f = filter ? filter_df4_resident_kernel<TB> : evolve_df4_resident_kernel<TB>;
+    const int smem = (filter ? 104 : 72) << TB;     // three or two vectors of 32 bytes a state, and the diagonal
     cudaError_t e = grow_smem_attr(reinterpret_cast<const void*>(f), smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -268,16 +384,16 @@ cudaError_t launch_df4_resident(const DfResArgs& a, int count, cudaStream_t st) 
 }  // namespace
 
 // Tiles of 2^10 or 2^11 states (the sizes of tile_step_df4x2 whose two vectors and diagonal fit shared
-// memory, 147 KB), at most 8 of them to a realization (a portable cluster).
+// memory: 147 KB, with the filter's third vector 213 KB), at most 8 of them to a realization (a portable cluster).
 bool df4_resident_fits(int tbits_uniform, int max_N) {
     return (tbits_uniform == 10 || tbits_uniform == 11) && max_N - tbits_uniform <= 3;
 }
 
-// Evolve the realizations a.list[0 .. count) in 2^a.lg CTAs each.
-cudaError_t launch_evolve_df4_resident(int tbits, const DfResArgs& a, int count, cudaStream_t st) {
+// Filter or evolve the realizations a.list[0 .. count) in 2^a.lg CTAs each.
+cudaError_t launch_df4_resident(int tbits, bool filter, const DfResArgs& a, int count, cudaStream_t st) {
     switch (tbits) {
-        case 10: return launch_df4_resident<10>(a, count, st);
-        case 11: return launch_df4_resident<11>(a, count, st);
+        case 10: return launch_df4_resident<10>(filter, a, count, st);
+        case 11: return launch_df4_resident<11>(filter, a, count, st);
     }
     return cudaErrorInvalidValue;
 }
