@@ -1101,6 +1101,20 @@ dacp_status choose_impl(dacp_ctx* c, int n_eigs, double d_ratio, double basis_ra
             bool redone = false;
             TRY(fx_launch(c, plan, q, em));
             TRY(fx_finish(c, q, em, &redone));
+        } else if (c->prec == kPrecDF32 && !c->has_pairs &&
+                   df1_resident_fits(c->tb_uniform, *std::max_element(c->N.begin(), c->N.end()))) {
+            TRY(resident_lists(c));
+            std::vector<int> list(R);
+            std::iota(list.begin(), list.end(), 0);
+            CK(cudaMemcpyAsync(c->fx_emax_d, em.data(), sizeof(double) * R, cudaMemcpyHostToDevice, c->st));
+            CK(cudaMemcpyAsync(c->fx_list_d, list.data(), sizeof(int) * R, cudaMemcpyHostToDevice, c->st));
+            DfResArgs q = df_resident_args(c);
+            q.list = c->fx_list_d;
+            q.psi = kA;
+            q.mom = kp;
+            CK(launch_moments_df1_resident(c->tb_uniform, q, R, *std::max_element(c->N.begin(), c->N.end()),
+                                           kpm_moments / 2, kpm_moments, c->st));
+            c->launches += 1;
         } else {
             c->launches += kpm_moments / 2;
             TRY(set_evolution_coef(c, em));

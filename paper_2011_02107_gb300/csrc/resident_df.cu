@@ -361,6 +361,127 @@ __global__ void __launch_bounds__(kDfThreads, 1) filter_df4_resident_kernel(cons
     }
 }
 
+// Moments of one column (the kernel-polynomial pre-pass): a CTA owns a realization, with both vectors and the
+// diagonal in shared memory, and no order needs more than the CTA's barrier. A slot holds two neighbouring
+// states. The bits are those of tile_step<df32, 1, kEvolve> on tiles of 2^TB states: the diagonal, then the
+// flips in rising bit order, the global flip, w_{k-1}; 256 running sums a tile, warps and tiles in order.
+// Bound by the float32 pipe: 190 paired instructions per two states and order. As 64 launches of one pass each,
+// 128 tiles of 64 sectors of 13 spins waited on L2 and on the tail of every launch: the parameter choice of the
+// sectors took 7.7 ms, and takes 4.8.
+template <int TB>
+__global__ void __launch_bounds__(kDfThreads, 1) moments_df1_resident_kernel(const DfResArgs a, const int orders,
+                                                                             const int rows_fixed) {
+    constexpr int kUnits = 1 << (TB - 1), U = kUnits / kThreads;     // slots of a tile, and of a thread
+    static_assert(U >= 1, "a tile gives every thread a slot");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) float4 gam_s[kMaxSpins + 1];
+    __shared__ __align__(8) float2 ngam_s[kMaxSpins + 1];
+    __shared__ double red_s[2][8][kThreads / 32][2];                 // [order parity][tile][warp][xx, ox]
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int r = a.list[blockIdx.x];
+    const RealInfo R = a.real[r];
+    const int slots = 1 << (R.N - 1), tiles = 1 << (R.N - TB);
+    ulonglong2* buf0 = reinterpret_cast<ulonglong2*>(smem_raw);
+    ulonglong2* buf1 = buf0 + slots;
+    ulonglong2* diag_s = buf1 + slots;                               // (d0.hi, d1.hi | d0.lo, d1.lo)
+    const Df4Fields gam{reinterpret_cast<const ulonglong2*>(gam_s), reinterpret_cast<const uint64_t*>(ngam_s)};
+    const bool gflip = a.gflip != nullptr;
+    const df32 ch = static_cast<df32>(2.0 / a.emax[r]);
+    const df32* psi = static_cast<const df32*>(a.psi) + R.off;
+    const df32* diag = a.diag + R.off;
+
+    df4_load_fields(gam_s, ngam_s, ch, a.gam + r * kMaxSpins, gflip ? a.gflip + r : nullptr, R.N);
+    auto pack = [](const df32 x, const df32 y) { return make_ulonglong2(pk2(x.hi, y.hi), pk2(x.lo, y.lo)); };
+    for (int i = tid; i < slots; i += blockDim.x) {
+        buf0[i] = pack(psi[2 * i], psi[2 * i + 1]);
+        diag_s[i] = pack(ch * diag[2 * i], ch * diag[2 * i + 1]);
+    }
+    __syncthreads();
+    double* mom = a.mom + static_cast<int64_t>(r) * rows_fixed;
+    auto write_row = [&](const int k) {                              // lanes 0, 1: rows 2 k, 2 k + 1
+        double tot = 0.0;
+        for (int t = 0; t < tiles; ++t) {
+            double s = 0.0;
+#pragma unroll
+            for (int w = 0; w < kThreads / 32; ++w) s += red_s[k & 1][t][w][lane];
+            tot += s;
+        }
+        mom[2 * k + lane] = tot;
+    };
+
+    for (int k = 0; k < orders; ++k) {
+        const ulonglong2* cur = (k & 1) ? buf1 : buf0;
+        ulonglong2* oth = (k & 1) ? buf0 : buf1;
+        auto at = [&](const int sl) {
+            const ulonglong2 v = cur[sl];
+            return DF2{v.x, v.y};
+        };
+        for (int t = tid / kThreads; t < tiles; t += blockDim.x / kThreads) {
+            const int base = t * kUnits + (tid & (kThreads - 1));
+            DF2 A[U];
+            Dot2x2 acc[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                A[u] = at(base + kThreads * u);
+                const ulonglong2 d = diag_s[base + kThreads * u];
+                acc[u] = dot2x2_prod(df2m(DF2{d.x, d.y}), A[u]);
+            }
+            {
+                const DF2m g = gam[0];
+#pragma unroll
+                for (int u = 0; u < U; ++u) dot2x2_mad(acc[u], g, df2_swap(A[u]));
+            }
+#pragma unroll 2
+            for (int i = 1; i < R.N; ++i) {
+                const DF2m g = gam[i];
+#pragma unroll
+                for (int u = 0; u < U; ++u) dot2x2_mad(acc[u], g, at((base + kThreads * u) ^ (1 << (i - 1))));
+            }
+            if (gflip) {
+                const DF2m g = gam[kMaxSpins];
+#pragma unroll
+                for (int u = 0; u < U; ++u) dot2x2_mad(acc[u], g, df2_swap(at((base + kThreads * u) ^ (slots - 1))));
+            }
+            Dot2x2 ms = Dot2x2{0ull, 0ull};                          // (<x, x> | <o, x>)
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int sl = base + kThreads * u;
+                if (k > 0) {
+                    const ulonglong2 y = oth[sl];
+                    dot2x2_sub(acc[u], DF2{y.x, y.y});
+                }
+                DF2 O = dot2x2_final(acc[u]);
+                if (k == 0) {
+                    const uint64_t half = pk2(0.5f, 0.5f);
+                    O = DF2{mul2(O.hi, half), mul2(O.lo, half)};
+                }
+                oth[sl] = make_ulonglong2(O.hi, O.lo);
+                const df32 x0 = df2_lane0(A[u]), x1 = df2_lane1(A[u]), o0 = df2_lane0(O), o1 = df2_lane1(O);
+                dot2x2_mad(ms, df2m(DF2{pk2(x0.hi, o0.hi), pk2(x0.lo, o0.lo)}), DF2{pk2(x0.hi, x0.hi), pk2(x0.lo, x0.lo)});
+                dot2x2_mad(ms, df2m(DF2{pk2(x1.hi, o1.hi), pk2(x1.lo, o1.lo)}), DF2{pk2(x1.hi, x1.hi), pk2(x1.lo, x1.lo)});
+            }
+            Dot2 s0, s1;
+            dot2x2_split(ms, s0, s1);
+            df32 v[2] = {dot2_final(s0), dot2_final(s1)};
+            const df32 sum = warp_reduce_scatter<2>(v, lane);
+            if ((lane & 15) == 0) red_s[k & 1][t][(tid & (kThreads - 1)) >> 5][lane >> 4] = static_cast<double>(sum);
+        }
+        __syncthreads();
+        if (tid >= static_cast<int>(blockDim.x) - 32 && lane < 2) write_row(k);    // beside the next order
+    }
+}
+
+template <int TB>
+cudaError_t launch_moments_df1(const DfResArgs& a, int count, int max_N, int orders, int rows_fixed, cudaStream_t st) {
+    auto* f = moments_df1_resident_kernel<TB>;
+    const int smem = 24 << max_N;
+    cudaError_t e = grow_smem_attr(reinterpret_cast<const void*>(f), smem);
+    if (e != cudaSuccess) return e;
+    f<<<count, max_N > TB ? kDfThreads : kThreads, smem, st>>>(a, orders, rows_fixed);
+    return cudaGetLastError();
+}
+
 template <int TB>
 cudaError_t launch_df4_resident(bool filter, const DfResArgs& a, int count, cudaStream_t st) {
     auto* f = filter ? filter_df4_resident_kernel<TB> : evolve_df4_resident_kernel<TB>;
@@ -394,6 +515,23 @@ cudaError_t launch_df4_resident(int tbits, bool filter, const DfResArgs& a, int 
     switch (tbits) {
         case 10: return launch_df4_resident<10>(filter, a, count, st);
         case 11: return launch_df4_resident<11>(filter, a, count, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// Tiles of 2^9 to 2^11 states, and two vectors and the diagonal of a realization (24 bytes a state) in the
+// shared memory of one CTA: up to 13 spins, in at most 8 tiles.
+bool df1_resident_fits(int tbits_uniform, int max_N) {
+    return tbits_uniform >= 9 && tbits_uniform <= 11 && max_N <= 13 && max_N - tbits_uniform <= 3;
+}
+
+// `orders` evolution orders of one column (a.psi) of the realizations a.list[0 .. count), rows at r * rows_fixed.
+cudaError_t launch_moments_df1_resident(int tbits, const DfResArgs& a, int count, int max_N, int orders, int rows_fixed,
+                                        cudaStream_t st) {
+    switch (tbits) {
+        case 9: return launch_moments_df1<9>(a, count, max_N, orders, rows_fixed, st);
+        case 10: return launch_moments_df1<10>(a, count, max_N, orders, rows_fixed, st);
+        case 11: return launch_moments_df1<11>(a, count, max_N, orders, rows_fixed, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -111,6 +111,27 @@ def test_double_float_clusters_keep_the_bits_of_the_per_order_launch(N, tile, fl
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("flip", [False, True])
+@pytest.mark.parametrize("N", [10, 11, 12, 13])
+def test_kpm_moments_of_one_cta_keep_the_bits_of_the_per_order_launch(N, flip):
+    """A 14-spin realization beside it takes the whole batch through the per-order launches: the parameters and
+    the features, which hold 32 of the moments, of the smaller one are equal to the last bit."""
+    models = [W.spin_glass_shard(n, seed=30 + n) for n in (N, 14)]
+    if flip:
+        models = [_flip(m, 0.6 - 0.1 * r) for r, m in enumerate(models)]
+    psis = [W.start_vectors(m["N"], 4, seed=9, r=r) for r, m in enumerate(models)]
+    out = []
+    for count in (1, 2):
+        d = P.Dacp(models[:count], psis[:count], block_b=4, precision=P.DACP_DF32)
+        try:
+            d.choose_params(20)
+            p = d.params()
+            out.append([np.asarray(p["a"])[0], np.asarray(p["emax"])[0], np.asarray(d.features())[0]])
+        finally:
+            d.close()
+    assert all(np.array_equal(x, y) for x, y in zip(*out))
+
+
 @pytest.mark.parametrize("name,prec,unit", PRECS)
 def test_bound_far_below_the_radius_is_reported_as_before(name, prec, unit):
     """Coefficients beyond the limbs, and vectors that outgrow the fixed point, end as DACP_ERR_NUMERIC."""
