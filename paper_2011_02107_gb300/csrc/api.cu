@@ -123,6 +123,15 @@ struct dacp_ctx {
     int emax_rule = 0;                  // E_max bound: 0 Ritz value + residual norm, 1 Ritz-residual rule
     double* mom_d = nullptr;
     int64_t mom_cap = 0;
+    // scratch of the parameter choice and of the read-backs, grown to the largest use up to kScratchKeep
+    void* scratch_d = nullptr;
+    size_t scratch_bytes = 0;
+    int* err_h = nullptr;               // pinned copy of err_d
+    // dacp_apply_h of float32 handles on the default tiles: a finer split (apply_geometry)
+    Item* apply_items_d = nullptr;
+    RealInfo* apply_info_d = nullptr;
+    std::vector<RealInfo> apply_info;
+    int apply_smem = 0;
     // fixed-point evolution (resident.cu): workspace, grown to the largest launch so far
     double* fx_emax_d = nullptr;        // [R]
     int *fx_list_d = nullptr, *fx_status_d = nullptr;   // [R]
@@ -253,6 +262,48 @@ void dfree(dacp_ctx* c, void* p) {
     if (it != c->allocs.end()) c->allocs.erase(it);
     cudaFree(p);
 }
+
+// Device scratch for the duration of one call: the handle's own up to kScratchKeep bytes (cudaMalloc and
+// cudaFree cost tens of microseconds each and wait for the device), an allocation of its own beyond.
+constexpr size_t kScratchKeep = 64 << 20;
+struct Scratch {
+    dacp_ctx* c;
+    char* p = nullptr;
+    size_t at = 0, size = 0;
+    bool own = false;
+    explicit Scratch(dacp_ctx* ctx) : c(ctx) {}
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    ~Scratch() {
+        if (own) dfree(c, p);
+    }
+    dacp_status reserve(size_t bytes) {
+        size = bytes;
+        if (bytes > kScratchKeep) {
+            void* v = nullptr;
+            TRY(dalloc(c, &v, bytes));
+            p = static_cast<char*>(v);
+            own = true;
+            return DACP_OK;
+        }
+        if (bytes > c->scratch_bytes) {
+            dfree(c, c->scratch_d);
+            c->scratch_d = nullptr;
+            c->scratch_bytes = 0;
+            TRY(dalloc(c, &c->scratch_d, bytes));
+            c->scratch_bytes = bytes;
+        }
+        p = static_cast<char*>(c->scratch_d);
+        return DACP_OK;
+    }
+    static size_t need(size_t bytes) { return (bytes + 255) & ~static_cast<size_t>(255); }
+    template <typename T>
+    T* take(size_t count) {
+        T* v = reinterpret_cast<T*>(p + at);
+        at += need(count * sizeof(T));
+        return v;
+    }
+};
 
 void free_lanes(dacp_ctx* c) {
     for (auto& L : c->lanes) {
@@ -414,8 +465,20 @@ dacp_status run_orders(dacp_ctx* c, bool filter, int orders,
     return DACP_OK;
 }
 
-// Work decomposition: tiles of at most tile_bytes of the vector per CTA.
+// Work decomposition: tiles of at most tile_bytes of the vector per CTA. The default tile of float64 handles
+// shrinks to 8 KB while the batch leaves SMs without one: the float64 pipe of the few SMs that had a tile bound
+// small batches (a 10-spin filter at b = 4: one CTA).
 void tile_geometry(dacp_ctx* c, int tile_bytes) {
+    c->tile_bytes = tile_bytes;
+    if (c->prec == kPrecF64 && tile_bytes == kTileBytes) {
+        auto tiles = [&](int bytes) {
+            int64_t n = 0;
+            for (int r = 0; r < c->R; ++r)
+                n += std::max<int64_t>(1, ((static_cast<int64_t>(c->b) * 8) << c->info[r].N) / bytes);
+            return n;
+        };
+        while (tile_bytes > kMinTileBytes && tiles(tile_bytes) < 152) tile_bytes /= 2;
+    }
     int tb_cap = 0;
     while ((static_cast<int64_t>(2) << tb_cap) * c->b * static_cast<int64_t>(c->esz) <= tile_bytes) ++tb_cap;
     c->items.clear();
@@ -429,7 +492,6 @@ void tile_geometry(dacp_ctx* c, int tile_bytes) {
         max_tstates = std::max(max_tstates, 1 << R.tbits);
     }
     c->smem = static_cast<int>(max_tstates * c->b * c->esz);
-    c->tile_bytes = tile_bytes;
     c->tb_uniform = c->R > 0 ? c->info[0].tbits : 0;
     for (int r = 1; r < c->R; ++r)
         if (c->info[r].tbits != c->tb_uniform) c->tb_uniform = 0;
@@ -444,6 +506,38 @@ size_t part_capacity(const dacp_ctx* c) {
         worst += static_cast<int64_t>(1) << (c->info[r].N - std::min(c->info[r].N, tb));
     }
     return static_cast<size_t>(std::max<int64_t>(worst, 1)) * 2 * c->b * c->b + 64;
+}
+
+// Float32 tiles of dacp_apply_h, which reads the vector once and keeps nothing: 1/128 of the vector, at least
+// 4 KB, at most 16 KB, against 64 KB for the recurrences, whose moments pay per tile. 16 KB and 64 KB tiles take
+// 26 and 37 us on 2^16 states at b = 4, 31 and 44 us on 2^18, 48 and 51 us on 2^20, call included. A tile
+// size that the caller set is kept.
+dacp_status apply_geometry(dacp_ctx* c) {
+    std::vector<Item> items;
+    c->apply_info = c->info;
+    const int64_t sv = static_cast<int64_t>(c->b) * static_cast<int64_t>(c->esz);      // bytes of a state
+    int max_states = 1;
+    for (int r = 0; r < c->R; ++r) {
+        RealInfo& R = c->apply_info[r];
+        const int64_t bytes = std::min<int64_t>(16384, std::max<int64_t>(4096, (sv << R.N) / 128));
+        int tb = 0;
+        while ((sv << (tb + 1)) <= bytes) ++tb;
+        R.tbits = std::min(R.N, std::max(tb, R.N - 10));         // at most the unrolled beyond-tile bits
+        while ((sv << R.tbits) > kTileBytes) --R.tbits;
+        R.item_begin = static_cast<int>(items.size());
+        R.item_count = 1 << (R.N - R.tbits);
+        for (int t = 0; t < R.item_count; ++t) items.push_back(Item{r, t});
+        max_states = std::max(max_states, 1 << R.tbits);
+    }
+    c->apply_smem = static_cast<int>(max_states * sv);
+    if (!c->apply_info_d) TRY(dalloc_t(c, &c->apply_info_d, static_cast<size_t>(c->R)));
+    Item* d = nullptr;
+    TRY(dalloc_t(c, &d, items.size()));
+    CK(cudaMemcpyAsync(c->apply_info_d, c->apply_info.data(), sizeof(RealInfo) * c->R, cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemcpyAsync(d, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    c->apply_items_d = d;
+    return DACP_OK;
 }
 
 // Switch the handle to a new tile size: items, smem attribute, graphs.
@@ -788,6 +882,7 @@ void dacp_destroy(dacp_handle c) {
     if (c->sol) cusolverDnDestroy(c->sol);
     if (c->blas) cublasDestroy(c->blas);
     for (void* p : c->allocs) cudaFree(p);
+    if (c->err_h) cudaFreeHost(c->err_h);
     if (c->own_stream && c->st) cudaStreamDestroy(c->st);
     delete c;
 }
@@ -921,6 +1016,8 @@ dacp_status dacp_create(dacp_handle* out, int n_real, const int* n_spins, const 
               ck(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st)) &&
               ck(cudaMemsetAsync(c->bar_d, 0, 2 * sizeof(unsigned), c->st));
     if (!ok) return bail(fail(c, DACP_ERR_CUDA, "upload failed"));
+    if (!ck(cudaMallocHost(&c->err_h, sizeof(int)))) return bail(fail(c, DACP_ERR_NOMEM, "pinned flag"));
+    if (c->fp32 && (s = apply_geometry(c)) != DACP_OK) return bail(s);
     // x-fields in the vector precision
     {
         if ((s = dalloc_t(c, &c->g64_d, c->g_h.size())) != DACP_OK) return bail(s);
@@ -1022,33 +1119,25 @@ dacp_status choose_impl(dacp_ctx* c, int n_eigs, double d_ratio, double basis_ra
     const int R = c->R;
     const int ni = static_cast<int>(c->items.size());
     const size_t sv = static_cast<size_t>(c->Dtot) * c->esz;   // one column
-    void *v0 = nullptr, *v1 = nullptr, *v2 = nullptr, *kA = nullptr, *kB = nullptr;
-    double *lmom = nullptr, *beta2 = nullptr, *emax_d = nullptr, *emax1_d = nullptr, *a_d = nullptr, *kp = nullptr;
-    int *K_d = nullptr, *n_d = nullptr;
-    float* knobs = nullptr;
-    auto cleanup = [&]() {
-        for (void* p : {v0, v1, v2, kA, kB, static_cast<void*>(lmom), static_cast<void*>(beta2),
-                        static_cast<void*>(emax_d), static_cast<void*>(emax1_d), static_cast<void*>(a_d),
-                        static_cast<void*>(kp),
-                        static_cast<void*>(K_d), static_cast<void*>(n_d), static_cast<void*>(knobs)})
-            dfree(c, p);
-    };
+    Scratch scr(c);
     auto run = [&]() -> dacp_status {
-        TRY(dalloc(c, &v0, sv));
-        TRY(dalloc(c, &v1, sv));
-        TRY(dalloc(c, &v2, sv));
-        TRY(dalloc(c, &kA, sv));
-        TRY(dalloc(c, &kB, sv));
         const int rows = 2 * steps;
-        TRY(dalloc_t(c, &lmom, static_cast<size_t>(R) * rows));
-        TRY(dalloc_t(c, &beta2, static_cast<size_t>(R) * steps));
-        TRY(dalloc_t(c, &emax_d, R));
-        TRY(dalloc_t(c, &emax1_d, R));
-        TRY(dalloc_t(c, &a_d, R));
-        TRY(dalloc_t(c, &kp, static_cast<size_t>(R) * kpm_moments));
-        TRY(dalloc_t(c, &K_d, R));
-        TRY(dalloc_t(c, &n_d, R));
-        TRY(dalloc_t(c, &knobs, static_cast<size_t>(R) * 3));
+        const size_t R8 = Scratch::need(sizeof(double) * R);
+        TRY(scr.reserve(5 * Scratch::need(sv) + Scratch::need(8 * static_cast<size_t>(R) * rows) +
+                        Scratch::need(8 * static_cast<size_t>(R) * steps) + 3 * R8 +
+                        Scratch::need(8 * static_cast<size_t>(R) * kpm_moments) + 2 * R8 +
+                        Scratch::need(4 * static_cast<size_t>(R) * 3)));
+        char *v0 = scr.take<char>(sv), *v1 = scr.take<char>(sv), *v2 = scr.take<char>(sv), *kA = scr.take<char>(sv),
+             *kB = scr.take<char>(sv);
+        double* lmom = scr.take<double>(static_cast<size_t>(R) * rows);
+        double* beta2 = scr.take<double>(static_cast<size_t>(R) * steps);
+        double* emax_d = scr.take<double>(R);
+        double* emax1_d = scr.take<double>(R);
+        double* a_d = scr.take<double>(R);
+        double* kp = scr.take<double>(static_cast<size_t>(R) * kpm_moments);
+        int* K_d = scr.take<int>(R);
+        int* n_d = scr.take<int>(R);
+        float* knobs = scr.take<float>(static_cast<size_t>(R) * 3);
         if (!c->feats_d) TRY(dalloc_t(c, &c->feats_d, static_cast<size_t>(R) * kFeatures));
         // v = column 0 of psi0, normalised; kept in kA for the KPM run
         CK(launch_extract_col(c->prec, c->b, c->psi0_d, v2, c->Dtot, c->st));
@@ -1164,9 +1253,7 @@ dacp_status choose_impl(dacp_ctx* c, int n_eigs, double d_ratio, double basis_ra
         c->n = nv;
         return apply_params(c);
     };
-    dacp_status s = run();
-    cleanup();
-    return s;
+    return run();
 }
 
 }  // namespace
@@ -1904,24 +1991,17 @@ dacp_status dacp_get_moments(dacp_handle c, int r, double* mu, int64_t cap, int6
     const int64_t nvals = static_cast<int64_t>(rows) * b * b;
     if (count) *count = nvals;
     if (cap < nvals) return fail(c, DACP_ERR_ARG, "capacity %lld < %lld", (long long)cap, (long long)nvals);
-    double *mus = nullptr, *nus = nullptr;
-    int* bad = nullptr;
-    auto run = [&]() -> dacp_status {
-        TRY(dalloc_t(c, &mus, static_cast<size_t>(nvals)));
-        TRY(dalloc_t(c, &nus, static_cast<size_t>(nvals)));
-        TRY(dalloc_t(c, &bad, 1));
-        CK(cudaMemsetAsync(bad, 0, sizeof(int), c->st));
-        CK(launch_moments(c->mom_d + c->info[r].mom_off * b * b, rows, b, c->emax[r], mus, nus, bad, c->st));
-        c->launches += 1;
-        CK(cudaMemcpyAsync(mu, mus, sizeof(double) * nvals, cudaMemcpyDeviceToHost, c->st));
-        CK(cudaStreamSynchronize(c->st));
-        return DACP_OK;
-    };
-    dacp_status s = run();
-    dfree(c, mus);
-    dfree(c, nus);
-    dfree(c, bad);
-    return s;
+    Scratch scr(c);
+    TRY(scr.reserve(2 * Scratch::need(sizeof(double) * nvals) + Scratch::need(sizeof(int))));
+    double* mus = scr.take<double>(static_cast<size_t>(nvals));
+    double* nus = scr.take<double>(static_cast<size_t>(nvals));
+    int* bad = scr.take<int>(1);
+    CK(cudaMemsetAsync(bad, 0, sizeof(int), c->st));
+    CK(launch_moments(c->mom_d + c->info[r].mom_off * b * b, rows, b, c->emax[r], mus, nus, bad, c->st));
+    c->launches += 1;
+    CK(cudaMemcpyAsync(mu, mus, sizeof(double) * nvals, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    return DACP_OK;
 }
 
 dacp_status dacp_get_filtered(dacp_handle c, int r, double* psi, int64_t cap) {
@@ -1930,19 +2010,15 @@ dacp_status dacp_get_filtered(dacp_handle c, int r, double* psi, int64_t cap) {
     if (r < 0 || r >= c->R || !psi) return fail(c, DACP_ERR_ARG, "bad realization or buffer");
     const int64_t n = (static_cast<int64_t>(1) << c->N[r]) * c->b;
     if (cap < n) return fail(c, DACP_ERR_ARG, "capacity too small");
-    double* tmp = nullptr;
-    auto run = [&]() -> dacp_status {
-        TRY(dalloc_t(c, &tmp, static_cast<size_t>(n)));
-        const char* src = static_cast<const char*>(c->psiE_d) + static_cast<size_t>(c->info[r].off) * c->b * c->esz;
-        CK(launch_to_double(c->prec, src, tmp, n, c->b, c->st));
-        c->launches += 1;
-        CK(cudaMemcpyAsync(psi, tmp, sizeof(double) * n, cudaMemcpyDeviceToHost, c->st));
-        CK(cudaStreamSynchronize(c->st));
-        return DACP_OK;
-    };
-    dacp_status s = run();
-    dfree(c, tmp);
-    return s;
+    Scratch scr(c);
+    TRY(scr.reserve(Scratch::need(sizeof(double) * n)));
+    double* tmp = scr.take<double>(static_cast<size_t>(n));
+    const char* src = static_cast<const char*>(c->psiE_d) + static_cast<size_t>(c->info[r].off) * c->b * c->esz;
+    CK(launch_to_double(c->prec, src, tmp, n, c->b, c->st));
+    c->launches += 1;
+    CK(cudaMemcpyAsync(psi, tmp, sizeof(double) * n, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    return DACP_OK;
 }
 
 }  // extern "C"
@@ -2364,10 +2440,20 @@ dacp_status dacp_apply_h(dacp_handle c, int r, const void* x_dev, void* y_dev) {
     a.x = static_cast<const char*>(x_dev) - shift;
     a.y1 = nullptr;
     a.out = static_cast<char*>(y_dev) - shift;
-    CK(launch_step(c->prec, c->b, kApply, a, c->info[r].item_begin, c->info[r].item_count, c->smem, c->st));
+    const RealInfo* info = &c->info[r];
+    int smem = c->smem;
+    if (c->fp32 && c->tile_bytes == kTileBytes) {
+        info = &c->apply_info[r];
+        smem = c->apply_smem;
+        a.items = c->apply_items_d;
+        a.real = c->apply_info_d;
+    }
+    CK(launch_step(c->prec, c->b, kApply, a, info->item_begin, info->item_count, smem, c->st));
     c->launches += 1;
+    // the flag of a wait that gave up comes back with the one synchronisation
+    CK(cudaMemcpyAsync(c->err_h, c->err_d, sizeof(int), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    return check_device_flag(c);
+    return *c->err_h ? check_device_flag(c) : DACP_OK;
 }
 
 // Bytes of the largest vector tile at tile_bytes (as tile_geometry sets c->smem).

@@ -146,3 +146,30 @@ def test_bound_far_below_the_radius_is_reported_as_before(name, prec, unit):
             assert (d.central_eigs(4)[1] == -4).all()
         finally:
             d.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("b,Ns", [(1, (1, 3, 8, 14, 17)), (2, (2, 9, 12, 16)), (4, (1, 5, 10, 13, 15, 18)), (4, (11,))])
+def test_apply_h_on_the_default_tiles(Ns, b, prec):
+    """Default tiles shrink with the batch (float64) and the vector (float32): every element within a rounding
+    per term, N flips, the global flip and the diagonal (itself summed from N (N + 1) / 2 terms), taken four
+    times, of the sum of the magnitudes."""
+    torch = pytest.importorskip("torch")
+    models = [_flip(W.random_model(N, seed=90 + i), 0.3 * (i % 2)) for i, N in enumerate(Ns)]
+    psis = [W.start_vectors(N, b, seed=13, r=i) for i, N in enumerate(Ns)]
+    f32 = prec == "fp32"
+    d = P.Dacp(models, psis, block_b=b, precision=P.DACP_FP32 if f32 else P.DACP_FP64)
+    try:
+        for r, m in enumerate(models):
+            N = m["N"]
+            xd = torch.from_numpy(np.ascontiguousarray(W.start_vectors(N, b, seed=14, r=r))).cuda()
+            xd = xd.float() if f32 else xd.double()
+            yd = torch.zeros_like(xd)
+            d.apply_h(r, xd.data_ptr(), yd.data_ptr())
+            x = xd.double().cpu().numpy()
+            ref, scale = Hm.apply_h_rows(m, x, np.arange(1 << N), with_abs=True)
+            dscale = (np.abs(np.triu(m["J"], 1)).sum() + np.abs(m["h"]).sum()) * np.abs(x)
+            tol = 4 * ((N + 4) * 2.0 ** (-24 if f32 else -53) * scale + (N * (N + 1) // 2 + 1) * 2.0 ** -53 * dscale)
+            assert (np.abs(yd.double().cpu().numpy() - ref) <= tol).all(), (r, N)
+    finally:
+        d.close()
