@@ -42,18 +42,18 @@ __device__ __forceinline__ float gemm_elem(const float* __restrict__ X, int ld, 
 // The network's layers are a few MFLOP, so latency bounds them: 32 x 32 tiles give 160 CTAs at a batch of
 // 640 and 256 wide layers, the next k tile is loaded under the current one's arithmetic, and the bias
 // gradient (rowsum) and the relu mask (gate) ride along instead of being launches of their own. Every value
-// sums in rising k, as a plain loop does. The 640-sample gradient takes 22 launches of 16 x 16 tiles with
-// one value a thread 378 us, host copies included.
+// sums in rising k, as a plain loop does. The 640-sample gradient, host copies included: 22 launches of
+// 16 x 16 tiles with one value a thread 378 us, these tiles 222, all weight gradients in one launch 163.
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(kGemmThreads) sgemm_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
-                                                             const float* __restrict__ B, int ldb, float* __restrict__ C,
-                                                             int ldc, const float* __restrict__ bias, int relu,
-                                                             const float* __restrict__ gate, float* __restrict__ rowsum) {
+__device__ __forceinline__ void gemm_tile(int bx, int by, int M, int N, int K, const float* __restrict__ A, int lda,
+                                          const float* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
+                                          const float* __restrict__ bias, int relu, const float* __restrict__ gate,
+                                          float* __restrict__ rowsum) {
     __shared__ float As[kTile][kTile + 2];       // [k][row], rows read in pairs
     __shared__ __align__(16) float Bs[kTile][kTile + 4];   // [k][column], columns read in fours
     constexpr int kLoads = kTile * kTile / kGemmThreads;
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    const int row0 = blockIdx.y * kTile, col0 = blockIdx.x * kTile;
+    const int row0 = by * kTile, col0 = bx * kTile;
     // neighbouring threads load neighbouring addresses: k runs fastest where it is contiguous
     const int ai = TA ? tid & 31 : tid >> 5, ak = TA ? tid >> 5 : tid & 31;
     const int bi = TB ? tid >> 5 : tid & 31, bk = TB ? tid & 31 : tid >> 5;
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kGemmThreads) sgemm_kernel(int M, int N, int K
     for (int i = 0; i < 2; ++i) {
         const int row = row0 + 2 * ty + i;
         if (row >= M) continue;
-        if (rowsum && blockIdx.x == 0 && tx == 0) rowsum[row] = sum[i];
+        if (rowsum && bx == 0 && tx == 0) rowsum[row] = sum[i];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int col = col0 + 4 * tx + j;
@@ -113,6 +113,35 @@ __global__ void __launch_bounds__(kGemmThreads) sgemm_kernel(int M, int N, int K
             C[at] = v;
         }
     }
+}
+
+template <bool TA, bool TB>
+__global__ void __launch_bounds__(kGemmThreads) sgemm_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
+                                                             const float* __restrict__ B, int ldb, float* __restrict__ C,
+                                                             int ldc, const float* __restrict__ bias, int relu,
+                                                             const float* __restrict__ gate) {
+    gemm_tile<TA, TB>(blockIdx.x, blockIdx.y, M, N, K, A, lda, B, ldb, C, ldc, bias, relu, gate, nullptr);
+}
+
+constexpr int kMaxLayers = 9;        // 8 hidden layers and the output
+
+struct GradArgs {
+    int layers, batch;
+    int first[kMaxLayers + 1];       // first block of each layer
+    int in[kMaxLayers], out[kMaxLayers];
+    const float *delta[kMaxLayers], *act[kMaxLayers];   // [batch][out], [batch][in]
+    float *w[kMaxLayers], *b[kMaxLayers];               // gradients: [out][in], [out]
+};
+
+// dW_l [out x in] = delta_l^T [out x batch] * a_l [batch x in] and db_l = sum of delta_l over the batch, of every
+// layer in one launch: a layer alone has too few tiles for the GPU (64 of 256 x 256 weights, 8 at the output)
+// and a serial sum over the batch, which bounds it (latency). The 640-sample gradient: 222 -> 163 us.
+__global__ void __launch_bounds__(kGemmThreads) weight_grads_kernel(const GradArgs g) {
+    int l = 0;
+    while (l + 1 < g.layers && static_cast<int>(blockIdx.x) >= g.first[l + 1]) ++l;
+    const int t = blockIdx.x - g.first[l], in = g.in[l], out = g.out[l], nx = (in + kTile - 1) / kTile;
+    gemm_tile<true, false>(t % nx, t / nx, out, in, g.batch, g.delta[l], out, g.act[l], in, g.w[l], in, nullptr, 0,
+                           nullptr, g.b[l]);
 }
 
 // delta = (y - t) / B, loss partials = (y - t)^2 / (2B)
@@ -172,9 +201,9 @@ __global__ void denorm_kernel(const float* __restrict__ z, int B, int F, const f
 
 template <bool TA, bool TB>
 static void sgemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-                  const float* bias, int relu, const float* gate, float* rowsum, cudaStream_t st) {
+                  const float* bias, int relu, const float* gate, cudaStream_t st) {
     dim3 grid((N + kTile - 1) / kTile, (M + kTile - 1) / kTile);
-    sgemm_kernel<TA, TB><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, relu, gate, rowsum);
+    sgemm_kernel<TA, TB><<<grid, kGemmThreads, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, relu, gate);
 }
 
 static int grid1(int64_t n) { return static_cast<int>(std::min<int64_t>((n + 255) / 256, 4096)); }
@@ -194,7 +223,7 @@ struct dacp_mlp_ctx {
     float *in_mean = nullptr, *in_std = nullptr, *out_mean = nullptr, *out_std = nullptr;
     float *out_lo = nullptr, *out_hi = nullptr;   // range the outputs are clamped to
     std::vector<float*> act;             // activations per layer, capacity cap_b rows
-    float* delta[2] = {nullptr, nullptr};
+    float* delta = nullptr;              // [batch][width] of every layer's output, one layer after the other
     float *xb = nullptr, *tb = nullptr, *yb = nullptr;
     double* loss_d = nullptr;
     int cap_b = 0;
@@ -221,25 +250,18 @@ dacp_status mfail(dacp_mlp_ctx* c, dacp_status s, const char* fmt, ...) {
         if (e_ != cudaSuccess) return mfail(c, DACP_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
     } while (0)
 
-int max_width(const dacp_mlp_ctx* c) {
-    int w = 0;
-    for (int s : c->sizes) w = std::max(w, s);
-    return w;
-}
-
 dacp_status ensure_batch(dacp_mlp_ctx* c, int B) {
     if (B <= c->cap_b) return DACP_OK;
     for (float* a : c->act) cudaFree(a);
-    cudaFree(c->delta[0]);
-    cudaFree(c->delta[1]);
+    cudaFree(c->delta);
     cudaFree(c->xb);
     cudaFree(c->tb);
     cudaFree(c->yb);
     c->act.assign(c->sizes.size(), nullptr);
-    const int W = max_width(c);
+    int64_t W = 0;
+    for (size_t l = 1; l < c->sizes.size(); ++l) W += c->sizes[l];
     for (size_t l = 0; l < c->sizes.size(); ++l) MCK(cudaMalloc(&c->act[l], sizeof(float) * B * c->sizes[l]));
-    MCK(cudaMalloc(&c->delta[0], sizeof(float) * B * W));
-    MCK(cudaMalloc(&c->delta[1], sizeof(float) * B * W));
+    MCK(cudaMalloc(&c->delta, sizeof(float) * B * W));
     MCK(cudaMalloc(&c->xb, sizeof(float) * B * c->sizes.front()));
     MCK(cudaMalloc(&c->tb, sizeof(float) * B * c->sizes.back()));
     MCK(cudaMalloc(&c->yb, sizeof(float) * B * c->sizes.back()));
@@ -253,7 +275,7 @@ void forward_dev(dacp_mlp_ctx* c, int B) {
     for (int l = 0; l < L; ++l) {
         const int in = c->sizes[l], out = c->sizes[l + 1];
         sgemm<false, true>(B, out, in, c->act[l], in, c->p + c->woff[l], in, c->act[l + 1], out,
-                           c->p + c->boff[l], l < L - 1 ? 1 : 0, nullptr, nullptr, c->st);
+                           c->p + c->boff[l], l < L - 1 ? 1 : 0, nullptr, c->st);
     }
     c->launches += L;
 }
@@ -262,24 +284,31 @@ void forward_dev(dacp_mlp_ctx* c, int B) {
 void backward_dev(dacp_mlp_ctx* c, int B) {
     const int L = static_cast<int>(c->sizes.size()) - 1;
     const int nout = c->sizes.back();
-    cudaMemsetAsync(c->loss_d, 0, sizeof(double), c->st);
-    mse_grad_kernel<<<grid1(B * nout), 256, 0, c->st>>>(c->act[L], c->tb, B * nout, 1.f / B, c->delta[0], c->loss_d);
-    c->launches += 1;
-    int cur = 0;
-    for (int l = L - 1; l >= 0; --l) {
-        const int in = c->sizes[l], out = c->sizes[l + 1];
-        // dW_l [out x in] = delta^T [out x B] * a_l [B x in], db_l = sum of delta over the batch
-        sgemm<true, false>(out, in, B, c->delta[cur], out, c->act[l], in, c->g + c->woff[l], in, nullptr, 0, nullptr,
-                           c->g + c->boff[l], c->st);
-        c->launches += 1;
-        if (l > 0) {
-            // delta_prev [B x in] = delta [B x out] * W_l [out x in], masked by relu' (z > 0 <=> a > 0)
-            sgemm<false, false>(B, in, out, c->delta[cur], out, c->p + c->woff[l], in, c->delta[1 - cur], in, nullptr,
-                                0, c->act[l], nullptr, c->st);
-            c->launches += 1;
-            cur = 1 - cur;
-        }
+    GradArgs g;
+    g.layers = L;
+    g.batch = B;
+    g.first[0] = 0;
+    float* at = c->delta;
+    float* delta[kMaxLayers];
+    for (int l = 0; l < L; ++l) {
+        delta[l] = at;
+        at += static_cast<int64_t>(B) * c->sizes[l + 1];
+        g.in[l] = c->sizes[l];
+        g.out[l] = c->sizes[l + 1];
+        g.delta[l] = delta[l];
+        g.act[l] = c->act[l];
+        g.w[l] = c->g + c->woff[l];
+        g.b[l] = c->g + c->boff[l];
+        g.first[l + 1] = g.first[l] + (g.in[l] + kTile - 1) / kTile * ((g.out[l] + kTile - 1) / kTile);
     }
+    cudaMemsetAsync(c->loss_d, 0, sizeof(double), c->st);
+    mse_grad_kernel<<<grid1(B * nout), 256, 0, c->st>>>(c->act[L], c->tb, B * nout, 1.f / B, delta[L - 1], c->loss_d);
+    // delta_{l-1} [B x in] = delta_l [B x out] * W_l [out x in], masked by relu' (z > 0 <=> a > 0)
+    for (int l = L - 1; l > 0; --l)
+        sgemm<false, false>(B, g.in[l], g.out[l], delta[l], g.out[l], c->p + c->woff[l], g.in[l], delta[l - 1], g.in[l],
+                            nullptr, 0, c->act[l], c->st);
+    weight_grads_kernel<<<g.first[L], kGemmThreads, 0, c->st>>>(g);
+    c->launches += L + 1;
 }
 
 }  // namespace
@@ -361,8 +390,8 @@ void dacp_mlp_destroy(dacp_mlp c) {
     for (void* q : {static_cast<void*>(c->p), static_cast<void*>(c->g), static_cast<void*>(c->m),
                     static_cast<void*>(c->v), static_cast<void*>(c->in_mean), static_cast<void*>(c->in_std),
                     static_cast<void*>(c->out_mean), static_cast<void*>(c->out_std), static_cast<void*>(c->out_lo),
-                    static_cast<void*>(c->out_hi), static_cast<void*>(c->delta[0]),
-                    static_cast<void*>(c->delta[1]), static_cast<void*>(c->xb), static_cast<void*>(c->tb),
+                    static_cast<void*>(c->out_hi), static_cast<void*>(c->delta),
+                    static_cast<void*>(c->xb), static_cast<void*>(c->tb),
                     static_cast<void*>(c->yb), static_cast<void*>(c->loss_d)})
         cudaFree(q);
     if (c->own_stream && c->st) cudaStreamDestroy(c->st);

@@ -190,3 +190,37 @@ def test_fallback_reruns_short_realizations_in_the_library():
         assert nf[r] == nref[r] == n_eigs and rank[r] == rref[r]
         assert np.array_equal(eigs[r], eref[r])
     assert all(4 * (2 * n + 1) < n_eigs for n in p_fb["n"])     # the handle keeps the learned run's state
+
+
+@pytest.mark.parametrize("batch", [1, 31, 64, 97])
+@pytest.mark.parametrize("n_in,width,layers,n_out", [(40, 256, 3, 3), (7, 33, 2, 5), (1, 1, 1, 1), (31, 8, 8, 65),
+                                                     (33, 1, 0, 32)])
+def test_gradients_of_all_layers_in_one_launch(n_in, width, layers, n_out, batch):
+    """Weights, inputs and targets of small whole numbers: every sum is exact in float32, and 1 / batch scales it
+    exactly where batch is a power of two. Elsewhere a rounding per term of the batch and of each layer."""
+    rng = np.random.default_rng(width + batch)
+    sizes = [n_in] + [width] * layers + [n_out]
+    params = []
+    for i, o in zip(sizes[:-1], sizes[1:]):
+        w = np.zeros((o, i))
+        for row in w:
+            row[rng.choice(i, min(i, 2), replace=False)] = rng.choice([-1.0, 1.0], min(i, 2))
+        params.append((w, rng.integers(-1, 2, o).astype(float)))
+    x = rng.integers(-2, 3, (batch, n_in)).astype(float)
+    t = rng.integers(-2, 3, (batch, n_out)).astype(float)
+    grads, loss_ref = OM.backward(params, x, t)
+    y, cache = OM.forward(params, x)
+    assert max(np.abs(c).max() for c in cache) * batch < 2 ** 20
+    delta, mags = np.abs(y - t) / batch, []
+    for l in reversed(range(layers + 1)):
+        mags.insert(0, (delta.T @ np.abs(cache[2 * l]), delta.sum(axis=0)))
+        delta = delta @ np.abs(params[l][0])
+    assert max(g.max() for pair in mags for g in pair) * batch < 2 ** 24
+    tol = 0.0 if batch & (batch - 1) == 0 else (batch + sum(sizes) + 2) * 2.0 ** -24 * OM.flatten(mags)
+    m = P.dacp_mlp_create(n_in, width, layers, n_out, weights=OM.flatten(params).astype(np.float32))
+    try:
+        g, loss = P.dacp_mlp_gradients(m, x.astype(np.float32), t.astype(np.float32), OM.flatten(grads).size)
+    finally:
+        P.dacp_mlp_destroy(m)
+    assert (np.abs(g - OM.flatten(grads)) <= tol).all()
+    assert abs(loss - loss_ref) <= 1e-6 * loss_ref
