@@ -102,8 +102,6 @@ def sector_inputs(wl, rank=0):
 # realizations of the default workload active, from one ncu capture of the current kernel (the
 # profile summaries keep the command); other workloads report none.
 DF32_EVOLVE_TRAFFIC = 316232448 + 101191936
-# the same for the launch over the 512 parity sectors (N - 1 = 13 spins) of that batch
-DF32_SECTOR_EVOLVE_TRAFFIC = 318150144 + 103256832
 DF32_TRAFFIC_SOURCE = "stored ncu capture of the current kernel, one launch, not re-measured in this run"
 # One error-free double-float multiply-add (the Dot2 step): TwoProduct 2,
 # TwoSum 6, and 4 float32 operations that fold the cross terms and the two
@@ -130,8 +128,9 @@ def roofline(wl, n_real, phase, bytes_evo, states_evo, clk, sms, launch_mode=0, 
     symmetric) double-float multiply-adds x DF_FMA_OPS float32 lane operations,
     plus b subtractions of w_{k-1} x DF_SUB_OPS, against the device's SMs x 128
     lanes x the SM clock sampled during the run.
-    float64: FP64-pipe bound; same multiply-add count against the measured
-    float64 dgemm rate (1.10 TFLOP/s = 0.55 T FMA/s on this GB300).
+    float64: the same multiply-add count against the measured float64 dgemm
+    rate (1.10 TFLOP/s = 0.55 T FMA/s on this GB300); the evolution runs in fixed
+    point on the integer pipe, so the fraction may exceed 1.
     sectors: the recurrences run on the parity sectors, N - 1 spins whose
     N - 1 x-fields and one global flip make N flip terms per state.
     """
@@ -148,7 +147,9 @@ def roofline(wl, n_real, phase, bytes_evo, states_evo, clk, sms, launch_mode=0, 
     df_ops_per_state = DF_FMA_OPS * (N * b + b + b * (b + 1)) + DF_SUB_OPS * b
     kern = {"fp32": "step_kernel<float,4,kEvolve>",
             "df32": "step_kernel_df4tb<kEvolve,11> (double-float, b = 4, paired float32 instructions)",
-            "fp64": "step_kernel<double,4,kEvolve>"}[wl["prec"]]
+            "fp64": f"evolve_fx_kernel<{b}> (59-bit fixed point on the integer pipe, vectors in shared memory)"}[wl["prec"]]
+    if wl["prec"] == "df32" and sectors and launch_mode == 0:
+        kern = "evolve_df4_resident_kernel<11> (double-float, b = 4, a cluster per sector, vectors in shared memory)"
     if wl["prec"] == "fp32":
         if launch_mode == 2:
             kern = "step_kernel_staged<4,kEvolve> (float32, x / w_{k-1} / diagonal tiles staged by bulk copies)"
@@ -159,8 +160,8 @@ def roofline(wl, n_real, phase, bytes_evo, states_evo, clk, sms, launch_mode=0, 
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                 "algorithmic": "3 * 2^N * b * 4 B per realization and order"}
     if wl["prec"] == "df32":
-        key = (N, b, n_real, bool(sectors))
-        traffic = {(14, 4, 256, False): DF32_EVOLVE_TRAFFIC, (14, 4, 512, True): DF32_SECTOR_EVOLVE_TRAFFIC}.get(key)
+        # the resident kernel of the sectors reads its vectors once a run
+        traffic = DF32_EVOLVE_TRAFFIC if (N, b, n_real, bool(sectors)) == (14, 4, 256, False) else None
         mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz") or 2070.0
         peak = sms * FP32_LANES_PER_SM * mhz * 1e6 / 1e12            # T lane-ops/s
         achieved = states_evo * df_ops_per_state / t_e / 1e12 if t_e > 0 else None

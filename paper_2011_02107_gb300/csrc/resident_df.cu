@@ -275,6 +275,9 @@ __global__ void __launch_bounds__(kDfThreads, 1) evolve_df4_resident_kernel(cons
 // The filter's recurrence w_{k+1} = 2 F w_k - w_{k-1}, F = (H^2 - E_c) / E_0 (Sec. II A), with w_k, w_{k-1}
 // (overwritten by w_{k+1}), u = H w_k and the diagonal resident: two passes and two cluster barriers an order.
 // w_K ends in pub0 (K even) or pub1 (K odd), as the per-order launch leaves it. pub0 holds w_0 at the start.
+// Bound by the float32 pipe, its issue and the last round of clusters: 500 orders of 64 sectors of 13 spins
+// (36 clusters at a time) take 22.2 ms, 29.4 as two launches an order; the filter of 512, 715 orders at most,
+// 149 and 166 ms.
 template <int TB>
 __global__ void __launch_bounds__(kDfThreads, 1) filter_df4_resident_kernel(const DfResArgs a) {
     constexpr int kSlots = 2 << TB, NI = kSlots / kDfThreads, U = NI < 4 ? NI : 4;
@@ -366,8 +369,8 @@ __global__ void __launch_bounds__(kDfThreads, 1) filter_df4_resident_kernel(cons
 // states. The bits are those of tile_step<df32, 1, kEvolve> on tiles of 2^TB states: the diagonal, then the
 // flips in rising bit order, the global flip, w_{k-1}; 256 running sums a tile, warps and tiles in order.
 // Bound by the float32 pipe: 190 paired instructions per two states and order. As 64 launches of one pass each,
-// 128 tiles of 64 sectors of 13 spins waited on L2 and on the tail of every launch: the parameter choice of the
-// sectors took 7.7 ms, and takes 4.8.
+// the 512 tiles of 128 sectors of 13 spins waited on L2 and on the tail of every launch: the parameter choice of
+// those sectors took 7.7 ms, and takes 4.8.
 template <int TB>
 __global__ void __launch_bounds__(kDfThreads, 1) moments_df1_resident_kernel(const DfResArgs a, const int orders,
                                                                              const int rows_fixed) {
@@ -521,6 +524,8 @@ cudaError_t launch_df4_resident(int tbits, bool filter, const DfResArgs& a, int 
 
 // Tiles of 2^9 to 2^11 states, and two vectors and the diagonal of a realization (24 bytes a state) in the
 // shared memory of one CTA: up to 13 spins, in at most 8 tiles.
+// Ahead at every batch size: the parameter choice of 1, 32, 152 and 512 sectors of 13 spins takes 3.5, 3.6, 4.2
+// and 10.4 ms with it, 4.3, 4.7, 7.5 and 19.8 without (and without the kept scratch).
 bool df1_resident_fits(int tbits_uniform, int max_N) {
     return tbits_uniform >= 9 && tbits_uniform <= 11 && max_N <= 13 && max_N - tbits_uniform <= 3;
 }
