@@ -372,6 +372,9 @@ dacp_status dacp_autotune(dacp_handle hd, int orders, int* tile_bytes_out);
  * (DACP_ERR_ARG), as is mode 2 on float64 or double-float vectors. Setting
  * resets filter and moment results. The resident evolution of DACP_FP64
  * handles (see dacp_basis_moments) does not depend on mode and tile size.
+ * At the default of 64 KB, DACP_FP64 handles split their vectors further, down
+ * to 8 KB, while the batch has fewer tiles than the GPU has SMs, and
+ * dacp_apply_h of DACP_FP32 handles uses tiles of 4 to 16 KB.
  */
 dacp_status dacp_set_launch(dacp_handle hd, int mode, int tile_bytes);
 dacp_status dacp_get_launch(dacp_handle hd, int* mode, int* tile_bytes);
