@@ -340,8 +340,9 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
         for (int e = 0; e < NT; ++e) ms[e].hh = ms[e].mm = 0;
         if (active) {
             for (int qb = 0; qb < q4; qb += nwork) {
+                if (qb + warp * 32 >= q4) break;         // a tile smaller than the CTA: no slot for this warp
                 const bool val = qb + tid < q4;
-                const int q = (qb + tid) & (q4 - 1);     // idle lanes repeat a slot and store nothing
+                const int q = (qb + tid) & (q4 - 1);     // idle lanes repeat a slot of their warp and store nothing
                 int4 x[U];
                 int64_t hh[U][2], mm[U][2];
 #pragma unroll
@@ -418,6 +419,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
                     fx_mad(hh[u][0], mm[u][0], d0, x[u].x, x[u].y);
                     fx_mad(hh[u][1], mm[u][1], d1, x[u].z, x[u].w);
                 }
+                __syncwarp();                            // the w_{k-1} of a repeated slot is read: it may be overwritten
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     int64_t o0 = (hh[u][0] << ge) + (mm[u][0] >> (29 - ge));

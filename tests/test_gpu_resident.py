@@ -173,3 +173,31 @@ def test_apply_h_on_the_default_tiles(Ns, b, prec):
             assert (np.abs(yd.double().cpu().numpy() - ref) <= tol).all(), (r, N)
     finally:
         d.close()
+
+
+@pytest.mark.parametrize("flip", [False, True])
+@pytest.mark.parametrize("b", [1, 2, 4])
+@pytest.mark.parametrize("Ns", [(3, 5, 13), (6, 9, 12, 7, 10)])
+def test_uneven_batches_have_the_moments_of_each_realization_alone(Ns, b, flip):
+    """Realizations with fewer slots than their CTA has threads, beside larger ones: the sums are exact integers, so
+    neither the number of CTAs nor that of threads shows in the moments, and none is declined (one launch)."""
+    models = [W.random_model(N, seed=110 + i) for i, N in enumerate(Ns)]
+    if flip:
+        models = [_flip(m, 0.37 * (-1) ** i) for i, m in enumerate(models)]
+    psis = [W.start_vectors(N, b, seed=15, r=i) for i, N in enumerate(Ns)]
+
+    def moments(at):
+        emax = np.array([_bound(models[i]) for i in at])
+        d = P.Dacp([models[i] for i in at], [psis[i] for i in at], block_b=b, precision=P.DACP_FP64)
+        try:
+            d.set_params(emax, 0.2 * emax, 0, 12)
+            d.filter()
+            before = d.launch_count()
+            d.basis_moments()
+            assert d.launch_count() == before + 1
+            return [d.moments(r) for r in range(len(at))]
+        finally:
+            d.close()
+
+    for i, mu in enumerate(moments(range(len(Ns)))):
+        assert np.array_equal(mu, moments([i])[0]), Ns[i]
