@@ -31,7 +31,7 @@ using namespace dacp;
 namespace {
 
 constexpr int kGraphOrders = 32;   // orders per captured graph
-constexpr int kMinTileBytes = 8192; // smallest tile the autotuner tries
+constexpr int kMinTileBytes = 8192; // smallest tile of the defaults and of the autotuner
 constexpr int kMaxLanes = 16;      // concurrent subspace solves
 constexpr double kLaneBytes = 24e9;  // device memory budget of the lanes
 // Float32 vectors: round-off in the recurrence leaves a noise floor near
@@ -112,6 +112,7 @@ struct dacp_ctx {
     void *gam_d = nullptr, *diag_d = nullptr;
     void *psi0_d = nullptr, *A_d = nullptr, *B_d = nullptr, *U_d = nullptr, *psiE_d = nullptr;
     double *coef_d = nullptr, *apply_coef_d = nullptr, *part_d = nullptr, *norms_d = nullptr;
+    size_t part_cap = 0;                // doubles of part_d
     unsigned *real_done_d = nullptr, *launch_done_d = nullptr;
     int* step_ctr_d = nullptr;
     int* err_d = nullptr;               // set by a stencil CTA whose bounded wait gave up
@@ -500,16 +501,8 @@ void tile_geometry(dacp_ctx* c, int tile_bytes) {
         if (c->info[r].tbits != c->tb_uniform) c->tb_uniform = 0;
 }
 
-// Partial-sum slots for the smallest tile the autotuner may pick.
-size_t part_capacity(const dacp_ctx* c) {
-    int64_t worst = 0;
-    for (int r = 0; r < c->R; ++r) {
-        int tb = 0;
-        while ((static_cast<int64_t>(2) << tb) * c->b * static_cast<int64_t>(c->esz) <= kMinTileBytes) ++tb;
-        worst += static_cast<int64_t>(1) << (c->info[r].N - std::min(c->info[r].N, tb));
-    }
-    return static_cast<size_t>(std::max<int64_t>(worst, 1)) * 2 * c->b * c->b + 64;
-}
+// Partial-sum slots of the present tiles: two b x b blocks each.
+size_t part_slots(const dacp_ctx* c) { return c->items.size() * 2 * c->b * c->b + 64; }
 
 // Float32 tiles of dacp_apply_h, which reads the vector once and keeps nothing: 1/128 of the vector, at least
 // 4 KB, at most 16 KB, against 64 KB for the recurrences, whose moments pay per tile. 16 KB and 64 KB tiles take
@@ -543,16 +536,37 @@ dacp_status apply_geometry(dacp_ctx* c) {
     return DACP_OK;
 }
 
-// Switch the handle to a new tile size: items, smem attribute, graphs.
+// Switch the handle to a new tile size: items, partial sums, smem attribute, graphs. A failure leaves the tiles
+// as they were.
 dacp_status retile(dacp_ctx* c, int tile_bytes) {
+    const int before = c->tile_bytes;
     tile_geometry(c, tile_bytes);
-    if (prepare_step(c->prec, c->b, c->smem) != cudaSuccess || prepare_step(c->prec, 1, c->smem) != cudaSuccess)
-        return fail(c, DACP_ERR_CUDA, "shared-memory attribute for %d bytes", c->smem);
-    if (c->launch_mode == 2 && prepare_step_staged(c->b, c->smem) != cudaSuccess)
-        return fail(c, DACP_ERR_CUDA, "staged shared-memory attribute for a %d-byte tile", c->smem);
+    Item* items = nullptr;
+    double* part = nullptr;
+    const size_t slots = part_slots(c);
+    auto make_room = [&]() -> dacp_status {
+        if (prepare_step(c->prec, c->b, c->smem) != cudaSuccess || prepare_step(c->prec, 1, c->smem) != cudaSuccess)
+            return fail(c, DACP_ERR_CUDA, "shared-memory attribute for %d bytes", c->smem);
+        if (c->launch_mode == 2 && prepare_step_staged(c->b, c->smem) != cudaSuccess)
+            return fail(c, DACP_ERR_CUDA, "staged shared-memory attribute for a %d-byte tile", c->smem);
+        TRY(dalloc_t(c, &items, c->items.size()));
+        if (slots > c->part_cap) TRY(dalloc_t(c, &part, slots));
+        return DACP_OK;
+    };
+    const dacp_status s = make_room();
+    if (s != DACP_OK) {
+        dfree(c, items);
+        dfree(c, part);
+        tile_geometry(c, before);
+        return s;
+    }
     dfree(c, c->items_d);
-    c->items_d = nullptr;
-    TRY(dalloc_t(c, &c->items_d, c->items.size()));
+    c->items_d = items;
+    if (part) {
+        dfree(c, c->part_d);
+        c->part_d = part;
+        c->part_cap = slots;
+    }
     CK(cudaMemcpyAsync(c->items_d, c->items.data(), sizeof(Item) * c->items.size(), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(c->info_d, c->info.data(), sizeof(RealInfo) * c->R, cudaMemcpyHostToDevice, c->st));
     CK(cudaStreamSynchronize(c->st));
@@ -999,7 +1013,8 @@ dacp_status dacp_create(dacp_handle* out, int n_real, const int* n_spins, const 
     ALLOC(dalloc(c, &c->psiE_d, vec_bytes));
     ALLOC(dalloc_t(c, &c->coef_d, 8 * static_cast<size_t>(n_real)));
     ALLOC(dalloc_t(c, &c->apply_coef_d, 8 * static_cast<size_t>(n_real)));
-    ALLOC(dalloc_t(c, &c->part_d, part_capacity(c)));
+    ALLOC(dalloc_t(c, &c->part_d, part_slots(c)));
+    c->part_cap = part_slots(c);
     ALLOC(dalloc_t(c, &c->norms_d, static_cast<size_t>(n_real) * block_b));
     ALLOC(dalloc_t(c, &c->real_done_d, n_real));
     ALLOC(dalloc_t(c, &c->launch_done_d, 1));
