@@ -587,7 +587,7 @@ dacp_status dacp_get_features(dacp_handle hd, float* feats, int64_t cap);
  * them).
  *
  *   n_spins      N, 1 <= N <= 16; larger N returns DACP_ERR_ARG (the scratch
- *                array below holds 3 x 2^16 float64 states).
+ *                array below holds 4 x 2^16 float64 states).
  *   J, h, gamma  host arrays as in dacp_create for one realization (J is
  *                N x N row-major, only i<j read).
  *   emax         bound on |E|; G = H / emax.
@@ -596,12 +596,13 @@ dacp_status dacp_get_features(dacp_handle hd, float* feats, int64_t cap);
  *   n_orders     evolution orders k = 0 .. n_orders-1.
  *   mu_dev       device pointer, 2 * n_orders float64: on return
  *                mu_j = <psi| T_j(G) |psi>, j = 0 .. 2 n_orders - 1, from the
- *                same fused stencil kernel as dacp_basis_moments.
+ *                same evolution as dacp_basis_moments of a DACP_FP64 handle.
+ *                It may overlap psi_dev.
  *   stream       cudaStream_t or NULL. The call copies J, h, gamma and its
  *                run lengths from host memory into the scratch array on this
  *                stream, and waits for the stream before it returns.
  *
- * Scratch: one file-scope device array of about 1.6 MB (vectors, diagonal,
+ * Scratch: one file-scope device array of about 2.1 MB (vectors, diagonal,
  * couplings, partial sums, counters), held by every GPU that loads the
  * library until the process exits. The first call on a device does the
  * set-up: it looks up the array's address (cudaGetSymbolAddress) and raises

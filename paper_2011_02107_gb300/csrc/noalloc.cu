@@ -17,6 +17,7 @@
 
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdint.h>
 #include <string.h>
 
 #include <mutex>
@@ -47,7 +48,8 @@ constexpr int64_t kRegItems = kRegInfo + 32;              // Item[kNaMaxItems]
 constexpr int64_t kRegCount = kRegItems + kNaMaxItems + 32;     // counters (unsigned / int)
 constexpr int64_t kRegEmax = kRegCount + 32;              // E_max
 constexpr int64_t kRegPro = kRegEmax + 32;                // scale exchange of the resident evolution
-constexpr int64_t kNaTotal = kRegPro + (2 << kFxMaxLg);
+constexpr int64_t kRegPsi = kRegPro + (2 << kFxMaxLg);    // start vector, when the moments are written over it
+constexpr int64_t kNaTotal = kRegPsi + kNaStates;
 
 static_assert(sizeof(RealInfo) <= 32 * sizeof(double), "RealInfo region too small");
 static_assert(sizeof(Item) * kNaMaxItems <= (kNaMaxItems + 32) * sizeof(double), "Item region too small");
@@ -139,6 +141,14 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
     const RealInfo* info_d = reinterpret_cast<const RealInfo*>(base + kRegInfo);
     if (launch_diag(kPrecF64, info_d, 0, N, base + kRegJ, base + kRegH, base + kRegDiag, st) != cudaSuccess)
         return DACP_ERR_CUDA;
+    // callers that count every byte may hand in overlapping buffers: the start vector is read after moments are written
+    const uintptr_t psi_at = reinterpret_cast<uintptr_t>(psi_dev), mu_at = reinterpret_cast<uintptr_t>(mu_dev);
+    const double* psi = psi_dev;
+    if (psi_at < mu_at + 2 * sizeof(double) * n_orders && mu_at < psi_at + sizeof(double) * D) {
+        if (!ok(cudaMemcpyAsync(base + kRegPsi, psi_dev, sizeof(double) * D, cudaMemcpyDeviceToDevice, st)))
+            return DACP_ERR_CUDA;
+        psi = base + kRegPsi;
+    }
 
     // the resident fixed-point evolution; what it does not suit (status word set) runs in floating point
     const int n = 2 * n_orders;
@@ -150,7 +160,7 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
         f.real = info_d;
         f.diag = base + kRegDiag;
         f.gam = base + kRegGam;
-        f.psi = psi_dev;
+        f.psi = psi;
         f.emax = base + kRegEmax;
         f.pub0 = reinterpret_cast<int4*>(base + kRegA);
         f.pub1 = reinterpret_cast<int4*>(base + kRegB);
@@ -171,7 +181,7 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
         if (!words[4]) return DACP_OK;
     }
     if (!ok(cudaMemsetAsync(counters + 4, 0, sizeof(unsigned), st)) ||
-        !ok(cudaMemcpyAsync(base + kRegA, psi_dev, sizeof(double) * D, cudaMemcpyDeviceToDevice, st)))
+        !ok(cudaMemcpyAsync(base + kRegA, psi, sizeof(double) * D, cudaMemcpyDeviceToDevice, st)))
         return DACP_ERR_CUDA;
     StepArgs a;
     memset(&a, 0, sizeof(a));

@@ -78,3 +78,28 @@ def test_noalloc_rejects_sizes_beyond_its_scratch():
     with pytest.raises(P.DacpError) as e:
         P.dacp_moments_noalloc(m, 10.0, x.data_ptr(), 4, x.data_ptr())
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("start", ["gauss", "one state", "even"])
+@pytest.mark.parametrize("shift", [0, 3, -7])
+@pytest.mark.parametrize("N", [8, 13])
+def test_moments_may_be_written_over_the_start_vector(N, shift, start):
+    """mu_dev at, behind and before psi_dev in one buffer; ordinary starts, and those the fixed-point evolution hands
+    on (a basis state) or may outgrow (all elements equal). The moments are those of separate buffers, to the bit."""
+    m = W.chain(N)
+    D = 1 << N
+    psi = {"gauss": W.start_vectors(N, 1, seed=1)[:, 0], "one state": np.eye(D)[5], "even": np.ones(D)}[start]
+    psi = psi / np.linalg.norm(psi)
+    orders = D // 4
+    emax = Hm.pauli_norm_bound(m)
+    buf = torch.zeros(16 + 2 * D, dtype=torch.float64, device="cuda")
+    sep = torch.zeros(2 * orders, dtype=torch.float64, device="cuda")
+    buf[16:16 + D] = torch.from_numpy(psi).cuda()
+    torch.cuda.synchronize()
+    x = buf[16:].data_ptr()
+    P.dacp_moments_noalloc(m, emax, x, orders, sep.data_ptr())
+    P.dacp_moments_noalloc(m, emax, x, orders, x + 8 * shift)
+    got = buf[16 + shift:16 + shift + 2 * orders]
+    assert torch.equal(got, sep), (got - sep).abs().max()
+    mu_or, _ = DA.chebyshev_moments(m, psi, emax, 2 * orders - 1)
+    assert np.abs(sep.cpu().numpy() - mu_or[:, 0, 0]).max() < 1e-9
