@@ -340,9 +340,9 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
         for (int e = 0; e < NT; ++e) ms[e].hh = ms[e].mm = 0;
         if (active) {
             for (int qb = 0; qb < q4; qb += nwork) {
-                if (qb + warp * 32 >= q4) break;         // a tile smaller than the CTA: no slot for this warp
                 const bool val = qb + tid < q4;
-                const int q = (qb + tid) & (q4 - 1);     // idle lanes repeat a slot of their warp and store nothing
+                const int q = (qb + tid) & (q4 - 1);     // idle lanes repeat a slot of w_k, and store and check nothing
+                const int4* old = val ? oth : cur;       // a repeated slot of w_{k-1} is being overwritten
                 int4 x[U];
                 int64_t hh[U][2], mm[U][2];
 #pragma unroll
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
                 if (k > 0) {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const int4 y = oth[u * q4 + q];
+                        const int4 y = old[u * q4 + q];
                         hh[u][0] += static_cast<int64_t>(y.x) * yone;
                         mm[u][0] += static_cast<int64_t>(y.y) * yone;
                         hh[u][1] += static_cast<int64_t>(y.z) * yone;
@@ -419,7 +419,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
                     fx_mad(hh[u][0], mm[u][0], d0, x[u].x, x[u].y);
                     fx_mad(hh[u][1], mm[u][1], d1, x[u].z, x[u].w);
                 }
-                __syncwarp();                            // the w_{k-1} of a repeated slot is read: it may be overwritten
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     int64_t o0 = (hh[u][0] << ge) + (mm[u][0] >> (29 - ge));
@@ -428,14 +427,14 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
                         o0 = (o0 + 1) >> 1;
                         o1 = (o1 + 1) >> 1;
                     }
-                    // |o| < 2^58: the top bits of the high word are all sign
-                    chk |= (static_cast<uint32_t>(static_cast<uint64_t>(o0) >> 32) + (1u << 26)) & ~((1u << 27) - 1u);
-                    chk |= (static_cast<uint32_t>(static_cast<uint64_t>(o1) >> 32) + (1u << 26)) & ~((1u << 27) - 1u);
                     const int2 l0 = fx_limbs(o0), l1 = fx_limbs(o1);
                     const int4 o = make_int4(l0.x, l0.y, l1.x, l1.y);
                     if (val) {
                         oth[u * q4 + q] = o;
                         if (lgr > 0) pnew[u * q4 + q] = o;
+                        // |o| < 2^58: the top bits of the high word are all sign
+                        chk |= (static_cast<uint32_t>(static_cast<uint64_t>(o0) >> 32) + (1u << 26)) & ~((1u << 27) - 1u);
+                        chk |= (static_cast<uint32_t>(static_cast<uint64_t>(o1) >> 32) + (1u << 26)) & ~((1u << 27) - 1u);
                     }
                     if constexpr (B == 4) {
                         // columns 2h, 2h + 1 of a state sit in the thread, the other pair in lane ^ 1 (the sums
