@@ -207,8 +207,12 @@ dacp_status dacp_filter(dacp_handle hd);
  * vectors themselves are never stored (Appendix C). Requires dacp_filter.
  * Handles of DACP_FP64 without pair couplings whose realizations fit the shared
  * memory of up to 128 CTAs (2^18 states at b = 4) evolve them there in 59-bit
- * fixed point, which is at least as accurate as float64 vectors; realizations
- * it does not suit (an element above 16 times the root mean square, or E_max
+ * fixed point. Its last place is 2^-57 to 2^-58 of the largest element of
+ * psi_E, so the accuracy is that of float64 vectors in the norm, not in every
+ * element. Vectors that outgrow this scale, as even ones do (a product state,
+ * random signs), start again at one whose last place is 2^-53 to 2^-52 of the
+ * root mean square. Realizations that neither suits (an element above 16 times
+ * the root mean square, most of the norm gathering in a few states, or E_max
  * not a bound) use float64 vectors in device memory. DACP_DF32 handles with
  * b = 4, no pair couplings and uniform tiles of 2^10 or 2^11 states, at most 8
  * to a realization, keep them in the shared memory of one cluster in launch

@@ -686,21 +686,13 @@ struct FxRun {
     int mom_rows_fixed, nsteps_override;
 };
 
-// Queue the fixed-point evolution of every realization (longest run first) on the handle's stream;
-// fx_status_d then names those it did not suit. emax: host values, uploaded here.
-dacp_status fx_launch(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std::vector<double>& emax) {
-    TRY(fx_workspace(c, q.b, plan));
-    std::vector<int> order(c->R);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-        const int64_t wx = static_cast<int64_t>(q.nsteps_override > 0 ? 1 : c->info[x].ne) << c->N[x];
-        const int64_t wy = static_cast<int64_t>(q.nsteps_override > 0 ? 1 : c->info[y].ne) << c->N[y];
-        return wx > wy;
-    });
-    CK(cudaMemcpyAsync(c->fx_emax_d, emax.data(), sizeof(double) * c->R, cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(c->fx_list_d, order.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemsetAsync(c->fx_status_d, 0, sizeof(int) * c->R, c->st));
-    CK(cudaMemsetAsync(c->fx_bar_d, 0, sizeof(unsigned) * c->R, c->st));
+// Queue the fixed-point evolution of the realizations `list` (longest run first) on the handle's stream;
+// fx_status_d, by place in the list, then names those it did not suit. emax: on the device in fx_emax_d.
+dacp_status fx_queue(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std::vector<int>& list, bool coarse) {
+    const int n = static_cast<int>(list.size());
+    CK(cudaMemcpyAsync(c->fx_list_d, list.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemsetAsync(c->fx_status_d, 0, sizeof(int) * n, c->st));
+    CK(cudaMemsetAsync(c->fx_bar_d, 0, sizeof(unsigned) * n, c->st));
     FxArgs a;
     memset(&a, 0, sizeof(a));
     a.list = c->fx_list_d;
@@ -720,23 +712,51 @@ dacp_status fx_launch(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std
     a.err_flag = c->err_d;
     a.mom_rows_fixed = q.mom_rows_fixed;
     a.nsteps_override = q.nsteps_override;
-    CK(launch_evolve_fx(q.b, plan, a, c->R, c->st));
-    c->launches += plan.sync == kFxCounter ? (c->R + plan.groups - 1) / plan.groups : 1;
+    a.coarse = coarse ? 1 : 0;
+    CK(launch_evolve_fx(q.b, plan, a, n, c->st));
+    c->launches += plan.sync == kFxCounter ? (n + plan.groups - 1) / plan.groups : 1;
     return DACP_OK;
 }
 
-// Wait for a fixed-point run and evolve the realizations it did not suit with the floating-point
-// kernels, one after the other. Leaves the evolution's coefficients on the device if there were any
-// (*redone): the caller restores the filter's.
-dacp_status fx_finish(dacp_ctx* c, const FxRun& q, const std::vector<double>& emax, bool* redone) {
-    std::vector<int> bad(c->R);
-    CK(cudaMemcpyAsync(bad.data(), c->fx_status_d, sizeof(int) * c->R, cudaMemcpyDeviceToHost, c->st));
+// Wait for a fixed-point run of `list`: the realizations it left to the floating-point kernels are added to
+// `rest`, those that want the coarse scale to `outgrown`.
+dacp_status fx_collect(dacp_ctx* c, const std::vector<int>& list, std::vector<int>& outgrown, std::vector<int>& rest) {
+    std::vector<int> status(list.size());
+    CK(cudaMemcpyAsync(status.data(), c->fx_status_d, sizeof(int) * status.size(), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    *redone = false;
-    for (int r = 0; r < c->R; ++r) {
-        if (!bad[r]) continue;
-        if (!*redone) TRY(set_evolution_coef(c, emax));
-        *redone = true;
+    for (size_t i = 0; i < list.size(); ++i) {
+        if (status[i] == kFxUnsuited) rest.push_back(list[i]);
+        else if (status[i] >= kFxOutgrown) outgrown.push_back(list[i]);
+    }
+    return DACP_OK;
+}
+
+// Evolve every realization: in fixed point, at the coarse scale where the vectors outgrow the first one, and with
+// the floating-point kernels, one after the other, where neither suits. Leaves the evolution's coefficients on
+// the device if there were any of those (*redone): the caller restores the filter's.
+dacp_status fx_evolve(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std::vector<double>& emax, bool* redone) {
+    TRY(fx_workspace(c, q.b, plan));
+    std::vector<int> order(c->R);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        const int64_t wx = static_cast<int64_t>(q.nsteps_override > 0 ? 1 : c->info[x].ne) << c->N[x];
+        const int64_t wy = static_cast<int64_t>(q.nsteps_override > 0 ? 1 : c->info[y].ne) << c->N[y];
+        return wx > wy;
+    });
+    CK(cudaMemcpyAsync(c->fx_emax_d, emax.data(), sizeof(double) * c->R, cudaMemcpyHostToDevice, c->st));
+    std::vector<int> outgrown, rest;
+    TRY(fx_queue(c, plan, q, order, false));
+    TRY(fx_collect(c, order, outgrown, rest));
+    if (!outgrown.empty()) {
+        std::vector<int> again;
+        TRY(fx_queue(c, plan, q, outgrown, true));
+        TRY(fx_collect(c, outgrown, again, rest));
+        rest.insert(rest.end(), again.begin(), again.end());
+    }
+    *redone = !rest.empty();
+    if (rest.empty()) return DACP_OK;
+    TRY(set_evolution_coef(c, emax));
+    for (const int r : rest) {
         const size_t at = static_cast<size_t>(c->info[r].off) * q.b * c->esz;
         CK(cudaMemcpyAsync(static_cast<char*>(q.pub0) + at, static_cast<const char*>(q.psi) + at,
                            (static_cast<size_t>(q.b) << c->N[r]) * c->esz, cudaMemcpyDeviceToDevice, c->st));
@@ -752,7 +772,7 @@ dacp_status fx_finish(dacp_ctx* c, const FxRun& q, const std::vector<double>& em
             CK(launch_step(c->prec, q.b, kEvolve, a, c->info[r].item_begin, c->info[r].item_count, c->smem, c->st));
         c->launches += orders;
     }
-    if (*redone) CK(cudaStreamSynchronize(c->st));
+    CK(cudaStreamSynchronize(c->st));
     return DACP_OK;
 }
 
@@ -1206,8 +1226,7 @@ dacp_status choose_impl(dacp_ctx* c, int n_eigs, double d_ratio, double basis_ra
         if (fx_usable(c, 1, &plan)) {
             const FxRun q{1, kA, kB, v0, kp, kpm_moments, kpm_moments / 2};
             bool redone = false;
-            TRY(fx_launch(c, plan, q, em));
-            TRY(fx_finish(c, q, em, &redone));
+            TRY(fx_evolve(c, plan, q, em, &redone));
         } else if (c->prec == kPrecDF32 && !c->has_pairs &&
                    df1_resident_fits(c->tb_uniform, *std::max_element(c->N.begin(), c->N.end()))) {
             TRY(resident_lists(c));
@@ -1351,8 +1370,7 @@ dacp_status dacp_basis_moments(dacp_handle c) {
     if (fx_usable(c, c->b, &plan)) {
         const FxRun q{c->b, c->psiE_d, c->A_d, c->B_d, c->mom_d, 0, 0};
         CK(cudaEventRecord(c->ev[2], c->st));
-        TRY(fx_launch(c, plan, q, c->emax));
-        TRY(fx_finish(c, q, c->emax, &coef));
+        TRY(fx_evolve(c, plan, q, c->emax, &coef));
     } else if (df_resident_usable(c)) {
         std::vector<int> order(c->R);
         std::iota(order.begin(), order.end(), 0);
@@ -1848,8 +1866,7 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
         if (fx_usable(c, b, &plan)) {
             const FxRun q{b, c->psiE_d, c->A_d, c->B_d, c->mom_d, 0, 0};
             CK(cudaEventRecord(c->ev[2], c->st));
-            TRY(fx_launch(c, plan, q, c->emax));
-            TRY(fx_finish(c, q, c->emax, &coef));
+            TRY(fx_evolve(c, plan, q, c->emax, &coef));
         } else if (df_resident_usable(c)) {
             // the groups that the per-order launch would hand over (their composition sets the padding of
             // the batched solves); each runs on a stream of its own, so that a group's solves start when

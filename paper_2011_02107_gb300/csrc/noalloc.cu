@@ -150,7 +150,8 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
         psi = base + kRegPsi;
     }
 
-    // the resident fixed-point evolution; what it does not suit (status word set) runs in floating point
+    // the resident fixed-point evolution, again at its coarse scale if the vectors outgrow the first; what neither
+    // suits runs in floating point
     const int n = 2 * n_orders;
     FxPlan plan;
     if (fx_plan(1, 1, N, N, &plan)) {
@@ -170,15 +171,19 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
         f.bar = counters + 4;
         f.status = reinterpret_cast<int*>(counters + 7);
         f.err_flag = reinterpret_cast<int*>(counters + 3);
-        if (launch_evolve_fx(1, plan, f, 1, st) != cudaSuccess) return DACP_ERR_CUDA;
-        noalloc_moments_from_products<<<(n + 255) / 256, 256, 0, st>>>(mu_dev, n);
-        unsigned words[5];                   // error flag .. status
-        if (cudaGetLastError() != cudaSuccess ||
-            !ok(cudaMemcpyAsync(words, counters + 3, sizeof(words), cudaMemcpyDeviceToHost, st)) ||
-            !ok(cudaStreamSynchronize(st)))
-            return DACP_ERR_CUDA;
-        if (words[0]) return DACP_ERR_TIMEOUT;
-        if (!words[4]) return DACP_OK;
+        for (f.coarse = 0; f.coarse < 2; ++f.coarse) {
+            if (f.coarse && !ok(cudaMemsetAsync(counters + 3, 0, 5 * sizeof(unsigned), st))) return DACP_ERR_CUDA;
+            if (launch_evolve_fx(1, plan, f, 1, st) != cudaSuccess) return DACP_ERR_CUDA;
+            noalloc_moments_from_products<<<(n + 255) / 256, 256, 0, st>>>(mu_dev, n);
+            unsigned words[5];                   // error flag .. status
+            if (cudaGetLastError() != cudaSuccess ||
+                !ok(cudaMemcpyAsync(words, counters + 3, sizeof(words), cudaMemcpyDeviceToHost, st)) ||
+                !ok(cudaStreamSynchronize(st)))
+                return DACP_ERR_CUDA;
+            if (words[0]) return DACP_ERR_TIMEOUT;
+            if (words[4] == kFxDone) return DACP_OK;
+            if (words[4] == kFxUnsuited) break;
+        }
     }
     if (!ok(cudaMemsetAsync(counters + 4, 0, sizeof(unsigned), st)) ||
         !ok(cudaMemcpyAsync(base + kRegA, psi, sizeof(double) * D, cudaMemcpyDeviceToDevice, st)))

@@ -53,10 +53,13 @@ struct FxArgs {
     longlong2* part;                // [groups][4][sums] moment sums in flight: x 2^24 + y
     double* mom;
     unsigned* bar;                  // [groups] barrier counters, zero (kFxCounter)
-    int* status;                    // [R] set to 1: evolve this realization in floating point
+    int* status;                    // [list] 0 at the start, an FxStatus at the end
     int* err_flag;
     int lg, sync, slots_max, mom_rows_fixed, nsteps_override;
+    int coarse;                     // 1: the scale with the most room (kFxOutgrown at the other one)
 };
+// kFxUnsuited: evolve this realization in floating point; above it: its vectors outgrew the scale.
+enum FxStatus { kFxDone = 0, kFxUnsuited = 1, kFxOutgrown = 2 };
 int fx_part_sums(int b);            // elements of FxArgs::part per group
 bool fx_plan(int b, int count, int minN, int maxN, FxPlan* p);
 cudaError_t launch_evolve_fx(int b, const FxPlan& p, const FxArgs& a, int count, cudaStream_t st);

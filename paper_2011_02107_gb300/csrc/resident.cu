@@ -21,10 +21,15 @@
 // 8 times its root mean square; moments of 2000 orders at 10 spins come out
 // 3 times, the amplified noise of their residual norms 20 times closer to an
 // 80-bit evaluation than in float64.
-// Realizations that this does not suit leave status[r] = 1 and are evolved by
-// the floating-point kernels: a vector with an element above 16 times its root
-// mean square, or one that outgrows 2^58 (E_max not a bound, or an element
-// that doubles its initial maximum), or couplings beyond the limbs.
+// The scale leaves 2 to 4 times the largest element as room. Random vectors
+// stay inside; one whose elements are even (a product state, random signs)
+// may concentrate and outgrow it, within some ten orders: the group then leaves
+// the run (status kFxOutgrown) and is launched again with room for 32 to 64
+// times the root mean square, the coarsest scale that any vector is given.
+// Realizations that this does not suit leave status kFxUnsuited and are evolved
+// by the floating-point kernels: a vector with an element above 16 times its
+// root mean square, one that outgrows the coarse scale as well (E_max not a
+// bound, or most of the norm in a few states), or couplings beyond the limbs.
 
 #include <math.h>
 
@@ -42,6 +47,7 @@ namespace {
 
 constexpr int kFxMinTileBits = 3;      // states of a tile: at least 2^3 (fewer CTAs of the group work below that)
 constexpr int kFxRedRing = 3, kFxPartRing = 4;   // orders in flight between a sum and its moment row
+constexpr int kFxCheck = 32;           // orders between two looks at the overflow flag
 constexpr uint64_t kFxWaitNs = 1000000000ull;
 
 template <int B> struct FxSums { static constexpr int value = B == 4 ? 20 : (B == 2 ? 6 : 2); };
@@ -149,6 +155,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     __shared__ FxSum red_s[kFxRedRing][kFxThreads / 32][NS];
     __shared__ float pro_s[3][kFxThreads / 32];
     __shared__ float max_s[4];
+    __shared__ int stop_s;                         // the group's status, read once in kFxCheck orders
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nwork = blockDim.x, nwarps = nwork >> 5;
@@ -227,7 +234,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
         __syncthreads();
     }
     const float mx = max_s[0], md = max_s[1], ss = max_s[2];
-    const int sexp = mx > 0.f ? 57 - (ilogbf(mx) + 1) : 0;             // |x| < 2^(57 - sexp)
+    int sexp = mx > 0.f ? 57 - (ilogbf(mx) + 1) : 0;                   // |x| < 2^(57 - sexp)
     const double c2 = 2.0 / emax;
     double gsum;
     bool fits = isfinite(ss) && mx > 0.f && isfinite(md) &&
@@ -240,8 +247,14 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
         gsum = gs * c2;
         fits = fits && gsum < 7.9;
     }
+    if (fits && a.coarse) {
+        // 16 times the root mean square in the place of the largest element
+        const int fine = sexp;
+        sexp = 57 - (ilogb(16.0 * sqrt(static_cast<double>(ss) / (ldexp(1.0, R.N) * B))) + 1);
+        fits = sexp < fine;
+    }
     if (!fits) {                                    // the same at every CTA of the group
-        if (rank == 0 && tid == 0) a.status[r] = 1;
+        if (rank == 0 && tid == 0) a.status[group] = kFxUnsuited;
         return;
     }
     // coefficients in units of 2^-(58 - ge): as fine as the sum of their magnitudes allows (limbs and 64-bit sums)
@@ -308,6 +321,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     // while order k's barrier is open: the CTA's sums of order k - 1, and the rows of order k - 3, whose
     // partials every CTA wrote before barrier k - 1. The warp may run behind by one order, hence the rings.
     auto moments_behind = [&](const int k) {
+        if (lane == 31 && k % kFxCheck == 2) stop_s = __ldcg(a.status + group);    // as of order k - 3
         if (active && lane < NS && k >= 1 && k <= orders) {
             long long hi = 0, lo = 0;
             for (int w = 0; w < nwarps; ++w) {
@@ -330,7 +344,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     const bool gf = a.gflip != nullptr;
     const int yone = -(1 << (29 - ge));             // -1 in the units of the sums
     uint32_t chk = 0;
-    for (int k = 0; k < orders; ++k) {
+    auto order = [&](const int k) -> bool {
         const int4* cur = (k & 1) ? buf1 : buf0;
         int4* oth = (k & 1) ? buf0 : buf1;
         const int4* pcur = ((k & 1) ? a.pub1 : a.pub0) + pslot0;
@@ -494,9 +508,17 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
                 if ((lane & 15) == 0) red_s[k % kFxRedRing][warp][lane >> 4] = s;
             }
         }
-        if (!fx_group_sync(a, group, target += G, [&] { moments_behind(k); })) return;
+        return fx_group_sync(a, group, target += G, [&] { moments_behind(k); });
+    };
+    for (int k0 = 0; k0 < orders; k0 += kFxCheck) {
+        const int k1 = k0 + kFxCheck < orders ? k0 + kFxCheck : orders;
+        for (int k = k0; k < k1; ++k)
+            if (!order(k)) return;
+        if (chk) a.status[group] = kFxOutgrown;
+        // the flag as it stood before this stretch (moments_behind), the same at every CTA of the group: the stretch's
+        // own is seen in the next one. (A look at every order takes 0.1 to 0.5 us of its 2 to 3.)
+        if (k0 > 0 && stop_s) return;
     }
-    if (chk) a.status[r] = 1;
     for (int k = orders; k < orders + 3; ++k)
         if (!fx_group_sync(a, group, target += G, [&] { moments_behind(k); })) return;
 }
@@ -586,6 +608,7 @@ cudaError_t launch_evolve_fx(int b, const FxPlan& p, const FxArgs& args, int cou
         FxArgs c = a;
         c.list = a.list + g0;
         c.bar = a.bar + g0;
+        c.status = a.status + g0;
         c.pro = a.pro + (static_cast<int64_t>(g0) << p.lg);
         c.part = a.part + static_cast<int64_t>(g0) * fx_part_sums(b);
         cudaLaunchConfig_t cfg = {};

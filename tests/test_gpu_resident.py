@@ -201,3 +201,32 @@ def test_uneven_batches_have_the_moments_of_each_realization_alone(Ns, b, flip):
 
     for i, mu in enumerate(moments(range(len(Ns)))):
         assert np.array_equal(mu, moments([i])[0]), Ns[i]
+
+
+@pytest.mark.parametrize("b", [1, 2, 4])
+@pytest.mark.parametrize("N,flip", [(6, 0.0), (9, 0.0), (10, 0.4), (13, 0.0), (14, -0.3)])
+def test_even_start_vectors_stay_in_fixed_point(N, flip, b):
+    """Starts whose elements are all alike in size concentrate under the evolution and outgrow the first scale: the
+    uniform product state, random signs and a constant with one sign changed. The run starts again with more room
+    (one launch more), never in floating point (a launch per order)."""
+    D = 1 << N
+    rng = np.random.default_rng(N)
+    cols = np.stack([np.ones(D), rng.choice([-1.0, 1.0], D), np.where(np.arange(D) == D // 3, -1.0, 1.0),
+                     rng.choice([-1.0, 1.0], D)], axis=1)[:, :b]
+    models = [dict(W.chain(N), gflip=flip), _flip(W.spin_glass_shard(N, seed=160), flip)]
+    emax = np.array([_bound(m) for m in models])
+    d = P.Dacp(models, [cols, cols], block_b=b, precision=P.DACP_FP64)
+    try:
+        d.set_params(emax, 0.2 * emax, 0, 19)             # 298 orders
+        d.filter()
+        before = d.launch_count()
+        d.basis_moments()
+        assert d.launch_count() == before + 2
+        kn = d.params()["kn"]
+        for r, m in enumerate(models):
+            mu = d.moments(r)
+            ref, _ = DA.chebyshev_moments(m, d.filtered(r), emax[r], mu.shape[0] - 1)
+            ref = 0.5 * (ref + ref.transpose(0, 2, 1))
+            assert np.abs(mu - ref).max() <= 8 * (N + 8) * 2.0 ** -53 * (kn[r] + 2) ** 2, r
+    finally:
+        d.close()
