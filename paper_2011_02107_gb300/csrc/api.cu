@@ -400,10 +400,43 @@ StepArgs base_args(dacp_ctx* c) {
     return a;
 }
 
+// Launch `orders` orders on the handle stream, `launches` stencil launches each. A graph of kGraphOrders of them is
+// captured once into g and replayed; realizations whose run is shorter skip the surplus orders inside the kernel.
+dacp_status replay_orders(dacp_ctx* c, Graph& g, int orders, int launches, const std::function<cudaError_t()>& launch_order,
+                          const std::function<dacp_status(int)>& after = std::function<dacp_status(int)>()) {
+    if (!g.exec && orders >= kGraphOrders) {
+        cudaGraph_t graph = nullptr;
+        CK(cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
+        cudaError_t le = cudaSuccess;
+        for (int i = 0; i < kGraphOrders && le == cudaSuccess; ++i) le = launch_order();
+        cudaError_t ee = cudaStreamEndCapture(c->st, &graph);
+        if (le != cudaSuccess) {
+            if (graph) cudaGraphDestroy(graph);
+            return fail(c, DACP_ERR_CUDA, "stencil launch during capture: %s", cudaGetErrorString(le));
+        }
+        CK(ee);
+        cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
+        cudaGraphDestroy(graph);
+        CK(ie);
+    }
+    int done = 0;
+    if (g.exec) {
+        for (; done + kGraphOrders <= orders; done += kGraphOrders) {
+            CK(cudaGraphLaunch(g.exec, c->st));
+            c->launches += kGraphOrders * launches;
+            if (after) TRY(after(done + kGraphOrders));
+        }
+    }
+    for (; done < orders; ++done) {
+        CK(launch_order());
+        c->launches += launches;
+        if (after) TRY(after(done + 1));
+    }
+    return DACP_OK;
+}
+
 // Launch `orders` Chebyshev orders of the filter (two stencil passes each) or of
-// the evolution (one pass each) on the handle stream. A graph of kGraphOrders
-// orders is captured once and replayed; realizations whose run is shorter
-// skip the surplus orders inside the kernel.
+// the evolution (one pass each) on the handle stream.
 dacp_status run_orders(dacp_ctx* c, bool filter, int orders,
                        const std::function<dacp_status(int)>& after = std::function<dacp_status(int)>()) {
     if (orders <= 0) return DACP_OK;
@@ -434,36 +467,7 @@ dacp_status run_orders(dacp_ctx* c, bool filter, int orders,
         }
         return pass(kEvolve);
     };
-    Graph& g = filter ? c->gf : c->ge;
-    if (!g.exec && orders >= kGraphOrders) {
-        cudaGraph_t graph = nullptr;
-        CK(cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
-        cudaError_t le = cudaSuccess;
-        for (int i = 0; i < kGraphOrders && le == cudaSuccess; ++i) le = launch_order();
-        cudaError_t ee = cudaStreamEndCapture(c->st, &graph);
-        if (le != cudaSuccess) {
-            if (graph) cudaGraphDestroy(graph);
-            return fail(c, DACP_ERR_CUDA, "stencil launch during capture: %s", cudaGetErrorString(le));
-        }
-        CK(ee);
-        cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
-        cudaGraphDestroy(graph);
-        CK(ie);
-    }
-    int done = 0;
-    if (g.exec) {
-        for (; done + kGraphOrders <= orders; done += kGraphOrders) {
-            CK(cudaGraphLaunch(g.exec, c->st));
-            c->launches += kGraphOrders * (filter ? 2 : 1);
-            if (after) TRY(after(done + kGraphOrders));
-        }
-    }
-    for (; done < orders; ++done) {
-        CK(launch_order());
-        c->launches += filter ? 2 : 1;
-        if (after) TRY(after(done + 1));
-    }
-    return DACP_OK;
+    return replay_orders(c, filter ? c->gf : c->ge, orders, filter ? 2 : 1, launch_order, after);
 }
 
 // Work decomposition: tiles of at most tile_bytes of the vector per CTA. The default tile of float64 handles
@@ -731,9 +735,59 @@ dacp_status fx_collect(dacp_ctx* c, const std::vector<int>& list, std::vector<in
     return DACP_OK;
 }
 
+// Evolve the realizations `rest` with the floating-point kernels: all of them in each order's launch, over the
+// tiles that are theirs. Leaves the evolution's coefficients on the device.
+dacp_status fx_redo(dacp_ctx* c, const FxRun& q, const std::vector<double>& emax, const std::vector<int>& rest) {
+    std::vector<RealInfo> info(c->info);
+    std::vector<Item> items;
+    int orders = 0;
+    for (const int r : rest) {
+        info[r].item_begin = static_cast<int>(items.size());
+        for (int t = 0; t < info[r].item_count; ++t) items.push_back(Item{r, t});
+        orders = std::max(orders, q.nsteps_override > 0 ? q.nsteps_override : info[r].ne);
+    }
+    RealInfo* info_d = nullptr;
+    Item* items_d = nullptr;
+    Graph g;
+    auto run = [&]() -> dacp_status {
+        TRY(dalloc_t(c, &info_d, info.size()));
+        TRY(dalloc_t(c, &items_d, items.size()));
+        TRY(set_evolution_coef(c, emax));
+        CK(cudaMemcpyAsync(info_d, info.data(), sizeof(RealInfo) * info.size(), cudaMemcpyHostToDevice, c->st));
+        CK(cudaMemcpyAsync(items_d, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice, c->st));
+        if (static_cast<int>(rest.size()) == c->R) {
+            CK(cudaMemcpyAsync(q.pub0, q.psi, static_cast<size_t>(c->Dtot) * q.b * c->esz, cudaMemcpyDeviceToDevice, c->st));
+        } else {
+            for (const int r : rest) {
+                const size_t at = static_cast<size_t>(info[r].off) * q.b * c->esz;
+                CK(cudaMemcpyAsync(static_cast<char*>(q.pub0) + at, static_cast<const char*>(q.psi) + at,
+                                   (static_cast<size_t>(q.b) << c->N[r]) * c->esz, cudaMemcpyDeviceToDevice, c->st));
+            }
+        }
+        CK(cudaMemsetAsync(c->step_ctr_d, 0, sizeof(int), c->st));
+        StepArgs a = base_args(c);
+        a.items = items_d;
+        a.real = info_d;
+        a.bufA = q.pub0;
+        a.bufB = q.pub1;
+        a.mom = q.mom;
+        a.mom_rows_fixed = q.mom_rows_fixed;
+        a.nsteps_override = q.nsteps_override;
+        const int ni = static_cast<int>(items.size());
+        TRY(replay_orders(c, g, orders, 1, [&] { return launch_step(c->prec, q.b, kEvolve, a, 0, ni, c->smem, c->st); }));
+        CK(cudaStreamSynchronize(c->st));
+        return DACP_OK;
+    };
+    const dacp_status s = run();
+    if (s != DACP_OK) cudaStreamSynchronize(c->st);
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    dfree(c, info_d);
+    dfree(c, items_d);
+    return s;
+}
+
 // Evolve every realization: in fixed point, at the coarse scale where the vectors outgrow the first one, and with
-// the floating-point kernels, one after the other, where neither suits. Leaves the evolution's coefficients on
-// the device if there were any of those (*redone): the caller restores the filter's.
+// the floating-point kernels where neither suits (*redone: the caller restores the filter's coefficients).
 dacp_status fx_evolve(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std::vector<double>& emax, bool* redone) {
     TRY(fx_workspace(c, q.b, plan));
     std::vector<int> order(c->R);
@@ -754,26 +808,7 @@ dacp_status fx_evolve(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std
         rest.insert(rest.end(), again.begin(), again.end());
     }
     *redone = !rest.empty();
-    if (rest.empty()) return DACP_OK;
-    TRY(set_evolution_coef(c, emax));
-    for (const int r : rest) {
-        const size_t at = static_cast<size_t>(c->info[r].off) * q.b * c->esz;
-        CK(cudaMemcpyAsync(static_cast<char*>(q.pub0) + at, static_cast<const char*>(q.psi) + at,
-                           (static_cast<size_t>(q.b) << c->N[r]) * c->esz, cudaMemcpyDeviceToDevice, c->st));
-        CK(cudaMemsetAsync(c->step_ctr_d, 0, sizeof(int), c->st));
-        StepArgs a = base_args(c);
-        a.bufA = q.pub0;
-        a.bufB = q.pub1;
-        a.mom = q.mom;
-        a.mom_rows_fixed = q.mom_rows_fixed;
-        a.nsteps_override = q.nsteps_override;
-        const int orders = q.nsteps_override > 0 ? q.nsteps_override : c->info[r].ne;
-        for (int k = 0; k < orders; ++k)
-            CK(launch_step(c->prec, q.b, kEvolve, a, c->info[r].item_begin, c->info[r].item_count, c->smem, c->st));
-        c->launches += orders;
-    }
-    CK(cudaStreamSynchronize(c->st));
-    return DACP_OK;
+    return rest.empty() ? DACP_OK : fx_redo(c, q, emax, rest);
 }
 
 // Whether the recurrences of launch mode 0 run as resident double-float clusters, one CTA per tile of the

@@ -230,3 +230,64 @@ def test_even_start_vectors_stay_in_fixed_point(N, flip, b):
             assert np.abs(mu - ref).max() <= 8 * (N + 8) * 2.0 ** -53 * (kn[r] + 2) ** 2, r
     finally:
         d.close()
+
+
+@pytest.mark.parametrize("b", [1, 4])
+def test_declined_realizations_run_side_by_side(b):
+    """Basis states (declined by the fixed point) beside ordinary blocks: one launch per order for all of them
+    together, as many as the longest takes, and nothing of the others' rows is touched."""
+    Ns = (10, 9, 11, 8, 12, 10)
+    declined = (0, 2, 3, 4)
+    models = [W.random_model(N, seed=170 + i) for i, N in enumerate(Ns)]
+    psis = [W.start_vectors(N, b, seed=18, r=i) for i, N in enumerate(Ns)]
+    for r in declined:
+        psis[r] = np.zeros_like(psis[r])
+        psis[r][3 + np.arange(b), np.arange(b)] = 1.0
+    emax = np.array([_bound(m) for m in models])
+    n = 4 + 2 * np.arange(len(Ns))
+    out = []
+    for at in (range(len(Ns)), [1], [5]):
+        d = P.Dacp([models[i] for i in at], [psis[i] for i in at], block_b=b, precision=P.DACP_FP64)
+        try:
+            d.set_params(emax[at], 0.2 * emax[at], 0, n[at])
+            d.filter()
+            before = d.launch_count()
+            d.basis_moments()
+            kn = d.params()["kn"]
+            longest = max([kn[r] + 2 for r in declined], default=0) if len(at) > 1 else 0
+            assert d.launch_count() == before + 1 + longest
+            out.append([d.moments(r) for r in range(len(at))])
+            if len(at) > 1:
+                for r in declined:
+                    ref, _ = DA.chebyshev_moments(models[r], d.filtered(r), emax[r], out[0][r].shape[0] - 1)
+                    ref = 0.5 * (ref + ref.transpose(0, 2, 1))
+                    tol = 8 * (Ns[r] + 8) * 2.0 ** -53 * (kn[r] + 2) ** 2
+                    assert np.abs(out[0][r] - ref).max() <= tol, r
+        finally:
+            d.close()
+    assert np.array_equal(out[0][1], out[1][0]) and np.array_equal(out[0][5], out[2][0])
+
+
+def test_window_of_declined_start_vectors():
+    """The 256 kernel-polynomial moments of a basis state come from the floating-point kernels, 128 launches for the
+    batch; the window agrees with the oracle's. An error e of the moments, at most 8 (N + 8) u 128^2 = 2.6e-10, moves
+    the level count by D e sum_j 4 / (pi j) < 2.1e-6 of 40, and the window by as much of itself."""
+    from oracle import params as OP
+    N, R = 10, 3
+    models = [W.spin_glass_shard(N, seed=180 + r) for r in range(R)]
+    one = np.zeros((1 << N, 2))
+    one[7, 0] = one[8, 1] = 1.0
+    launches, p = [], None
+    for psis in ([one] * R, [W.start_vectors(N, 2, seed=19, r=r) for r in range(R)]):
+        d = P.Dacp(models, psis, block_b=2, precision=P.DACP_FP64)
+        try:
+            before = d.launch_count()
+            d.choose_params(20)
+            launches.append(d.launch_count() - before)
+            p = p or d.params()
+        finally:
+            d.close()
+    assert launches[0] == launches[1] + 128
+    for r, m in enumerate(models):
+        mu = OP.kpm_moments(m, one[:, 0], p["emax"][r], 256)
+        assert abs(p["a"][r] / OP.kpm_window(mu, 1 << N, p["emax"][r], 40.0) - 1.0) < 1e-7, r
