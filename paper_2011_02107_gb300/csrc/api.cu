@@ -142,7 +142,9 @@ struct dacp_ctx {
     size_t fx_ctas = 0, fx_parts = 0;
     double* df_part_d = nullptr;        // double-float resident evolution (resident_df.cu): sums in flight
     size_t df_parts = 0;
-    std::vector<cudaStream_t> df_st;    // streams its groups run on beside each other (dacp_solve)
+    std::vector<cudaStream_t> df_st;    // streams its groups and sizes run on beside each other
+    std::vector<cudaEvent_t> df_ev;     // one each
+    cudaEvent_t df_fork = nullptr;
 
     // parameters
     std::vector<double> emax, a;
@@ -825,7 +827,6 @@ bool df_resident_usable(const dacp_ctx* c) {
 DfResArgs df_resident_args(const dacp_ctx* c) {
     DfResArgs a;
     memset(&a, 0, sizeof(a));
-    while (c->tb_uniform + a.lg < *std::max_element(c->N.begin(), c->N.end())) ++a.lg;
     a.real = c->info_d;
     a.diag = static_cast<const df32*>(c->diag_d);
     a.gam = static_cast<const df32*>(c->gam_d);
@@ -836,34 +837,55 @@ DfResArgs df_resident_args(const dacp_ctx* c) {
     a.pub0 = static_cast<ulonglong2*>(c->A_d);
     a.pub1 = static_cast<ulonglong2*>(c->B_d);
     a.pubu = static_cast<ulonglong2*>(c->U_d);
-    a.part = c->df_part_d;
     a.mom = c->mom_d;
     return a;
 }
 
-// Queue the filter's recurrence of every realization, w_0 in A, longest run first.
-dacp_status df_resident_filter(dacp_ctx* c) {
-    TRY(resident_lists(c));
-    std::vector<int> list(c->R);
-    std::iota(list.begin(), list.end(), 0);
-    std::stable_sort(list.begin(), list.end(), [&](int x, int y) { return c->K[x] > c->K[y]; });
-    CK(cudaMemcpyAsync(c->fx_list_d, list.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
-    DfResArgs a = df_resident_args(c);
-    a.list = c->fx_list_d;
-    CK(launch_df4_resident(c->tb_uniform, true, a, c->R, c->st));
-    c->launches += 1;
+// `count` streams beside the handle's own, each with an event.
+dacp_status df_resident_streams(dacp_ctx* c, size_t count) {
+    if (!c->df_fork) CK(cudaEventCreateWithFlags(&c->df_fork, cudaEventDisableTiming));
+    while (c->df_st.size() < count) {
+        cudaStream_t s = nullptr;
+        cudaEvent_t e = nullptr;
+        CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        c->df_ev.push_back(e);
+        CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+        c->df_st.push_back(s);
+    }
     return DACP_OK;
 }
 
-// Queue the resident double-float evolution of the realizations order[0 .. R), group by group: group g is
-// order[from[g] .. from[g + 1]) (from ends with R) and runs on stream st[g], in rising group order where
-// SMs are short and with the longest runs of a group first. psi_E, the two recurrence buffers and the moment
-// rows are the handle's.
-dacp_status df_resident_launch(dacp_ctx* c, const std::vector<int>& order, const std::vector<int>& from,
-                               const std::vector<cudaStream_t>& st) {
+// Queue the resident double-float filter (w_0 in A) or evolution (w_0 in psi_E) of the realizations
+// order[0 .. R), group by group: group g is order[from[g] .. from[g + 1]) (from ends with R) and is done when
+// done[g], a stream, is; done[0] is the handle's. Every size has a launch of its own, with clusters of as many
+// CTAs as it has tiles: 300 filter orders of 512 shards, half of them of 11 and half of 13 spins, take 50.6 ms,
+// 60.7 as per-order launches and 80.8 in clusters of the largest size's. The launches run on streams beside each other, in rising group order and falling size where SMs are short, the
+// longest runs of each first. The streams of groups 1, 2, ... are the first of the handle's extra ones.
+dacp_status df_resident_launch(dacp_ctx* c, bool filter, const std::vector<int>& order, const std::vector<int>& from,
+                               std::vector<cudaStream_t>* done) {
     TRY(resident_lists(c));
-    DfResArgs a = df_resident_args(c);
-    const size_t parts = (static_cast<size_t>(c->R) << a.lg) * kDfPartSums;
+    const int ng = static_cast<int>(from.size()) - 1;
+    struct Part {
+        int group, from, count, lg;
+    };
+    std::vector<Part> launches;
+    std::vector<int> list(order);
+    size_t ctas = 0;
+    for (int g = 0; g < ng; ++g) {
+        std::stable_sort(list.begin() + from[g], list.begin() + from[g + 1], [&](int x, int y) {
+            if (c->N[x] != c->N[y]) return c->N[x] > c->N[y];
+            return filter ? c->K[x] > c->K[y] : c->info[x].ne > c->info[y].ne;
+        });
+        for (int i = from[g]; i < from[g + 1];) {
+            int k = i;
+            while (k < from[g + 1] && c->N[list[k]] == c->N[list[i]]) ++k;
+            const int lg = std::max(0, c->N[list[i]] - c->tb_uniform);
+            launches.push_back(Part{g, i, k - i, lg});
+            ctas += static_cast<size_t>(k - i) << lg;
+            i = k;
+        }
+    }
+    const size_t parts = filter ? 0 : ctas * kDfPartSums;
     if (parts > c->df_parts) {
         dfree(c, c->df_part_d);
         c->df_part_d = nullptr;
@@ -871,32 +893,44 @@ dacp_status df_resident_launch(dacp_ctx* c, const std::vector<int>& order, const
         TRY(dalloc_t(c, &c->df_part_d, parts));
         c->df_parts = parts;
     }
-    const int ng = static_cast<int>(from.size()) - 1;
-    std::vector<int> list(order);
-    for (int g = 0; g < ng; ++g)
-        std::stable_sort(list.begin() + from[g], list.begin() + from[g + 1],
-                         [&](int x, int y) { return c->info[x].ne > c->info[y].ne; });
-    CK(cudaMemcpyAsync(c->fx_emax_d, c->emax.data(), sizeof(double) * c->R, cudaMemcpyHostToDevice, c->st));
+    TRY(df_resident_streams(c, launches.size() - 1));
+    done->assign(1, c->st);
+    done->insert(done->end(), c->df_st.begin(), c->df_st.begin() + (ng - 1));
+    if (!filter)
+        CK(cudaMemcpyAsync(c->fx_emax_d, c->emax.data(), sizeof(double) * c->R, cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync(c->fx_list_d, list.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
-    CK(cudaEventRecord(c->ev[2], c->st));            // also the start of T_E
-    for (int g = 0; g < ng; ++g) {
-        if (st[g] != c->st) CK(cudaStreamWaitEvent(st[g], c->ev[2], 0));
-        a.list = c->fx_list_d + from[g];
-        a.part = c->df_part_d + (static_cast<size_t>(from[g]) << a.lg) * kDfPartSums;
-        CK(launch_df4_resident(c->tb_uniform, false, a, from[g + 1] - from[g], st[g]));
+    if (launches.size() > 1) CK(cudaEventRecord(c->df_fork, c->st));
+    DfResArgs a = df_resident_args(c);
+    a.part = c->df_part_d;
+    int extra = ng - 1;                              // extra streams taken
+    for (size_t i = 0; i < launches.size(); ++i) {
+        const Part& p = launches[i];
+        const bool first = i == 0 || launches[i - 1].group != p.group;
+        const int at = first ? p.group - 1 : extra++;
+        cudaStream_t st = at < 0 ? c->st : c->df_st[at];
+        if (at >= 0) CK(cudaStreamWaitEvent(st, c->df_fork, 0));
+        a.list = c->fx_list_d + p.from;
+        a.lg = p.lg;
+        CK(launch_df4_resident(c->tb_uniform, filter, a, p.count, st));
         c->launches += 1;
+        a.part += (static_cast<size_t>(p.count) << p.lg) * kDfPartSums;
+        if (!first) {
+            CK(cudaEventRecord(c->df_ev[at], st));
+            CK(cudaStreamWaitEvent((*done)[p.group], c->df_ev[at], 0));
+        }
     }
     return DACP_OK;
 }
 
-// `count` streams beside the handle's own.
-dacp_status df_resident_streams(dacp_ctx* c, size_t count) {
-    while (c->df_st.size() < count) {
-        cudaStream_t s = nullptr;
-        CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-        c->df_st.push_back(s);
-    }
-    return DACP_OK;
+// The same for the whole batch on the handle's stream.
+dacp_status df_resident_run(dacp_ctx* c, bool filter) {
+    std::vector<int> order(c->R);
+    std::iota(order.begin(), order.end(), 0);
+    std::vector<cudaStream_t> done;
+    const dacp_status s = df_resident_launch(c, filter, order, {0, c->R}, &done);
+    if (s != DACP_OK)                                // what was queued beside the handle's stream must not outlive the call
+        for (cudaStream_t st : c->df_st) cudaStreamSynchronize(st);
+    return s;
 }
 
 dacp_status set_evolution_coef(dacp_ctx* c, const std::vector<double>& emax) {
@@ -941,6 +975,8 @@ void dacp_destroy(dacp_handle c) {
         cudaStreamSynchronize(s);
         cudaStreamDestroy(s);
     }
+    for (cudaEvent_t e : c->df_ev) cudaEventDestroy(e);
+    if (c->df_fork) cudaEventDestroy(c->df_fork);
     free_lanes(c);
     if (c->gf.exec) cudaGraphExecDestroy(c->gf.exec);
     if (c->ge.exec) cudaGraphExecDestroy(c->ge.exec);
@@ -1377,7 +1413,7 @@ dacp_status dacp_filter(dacp_handle c) {
     for (int r = 0; r < c->R; ++r) maxK = std::max(maxK, c->K[r]);
     CK(cudaEventRecord(c->ev[0], c->st));
     CK(cudaMemcpyAsync(c->A_d, c->psi0_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
-    if (df_resident_usable(c)) TRY(df_resident_filter(c));
+    if (df_resident_usable(c)) TRY(df_resident_run(c, true));
     else TRY(run_orders(c, true, maxK));
     // psi_E = w_K / |w_K| per column; w_K sits in A (K even) or B (K odd); also w_0 of the evolution
     c->launches += 2;
@@ -1407,9 +1443,8 @@ dacp_status dacp_basis_moments(dacp_handle c) {
         CK(cudaEventRecord(c->ev[2], c->st));
         TRY(fx_evolve(c, plan, q, c->emax, &coef));
     } else if (df_resident_usable(c)) {
-        std::vector<int> order(c->R);
-        std::iota(order.begin(), order.end(), 0);
-        TRY(df_resident_launch(c, order, {0, c->R}, {c->st}));
+        CK(cudaEventRecord(c->ev[2], c->st));
+        TRY(df_resident_run(c, false));
         coef = false;
     } else {
         TRY(set_evolution_coef(c, c->emax));
@@ -1916,10 +1951,9 @@ dacp_status dacp_solve(dacp_handle c, int n_eigs, double window, double eps, dou
             for (int done = maxE - maxE % kGraphOrders + 1; done <= maxE; ++done) TRY(after(done));
             if (from.back() < R) from.push_back(R);
             const size_t ng = from.size() - 1;
-            TRY(df_resident_streams(c, ng - 1));
-            std::vector<cudaStream_t> st(c->df_st.begin(), c->df_st.begin() + (ng - 1));
-            st.insert(st.begin(), c->st);
-            TRY(df_resident_launch(c, order, from, st));
+            std::vector<cudaStream_t> st;
+            CK(cudaEventRecord(c->ev[2], c->st));
+            TRY(df_resident_launch(c, false, order, from, &st));
             coef = false;
             dispatched = R;
             for (size_t g = 0; g < ng; ++g) TRY(push(order, from[g], from[g + 1], st[g]));

@@ -291,3 +291,36 @@ def test_window_of_declined_start_vectors():
     for r, m in enumerate(models):
         mu = OP.kpm_moments(m, one[:, 0], p["emax"][r], 256)
         assert abs(p["a"][r] / OP.kpm_window(mu, 1 << N, p["emax"][r], 40.0) - 1.0) < 1e-7, r
+
+
+@pytest.mark.parametrize("flip", [False, True])
+@pytest.mark.parametrize("Ns,tile", [((11, 13, 12, 13, 11, 12, 11), 65536), ((10, 12, 11, 13, 10), 32768),
+                                     ((11, 14, 12), 65536), ((12,) * 9, 65536)])
+def test_double_float_clusters_of_every_size_keep_the_bits(Ns, tile, flip):
+    """One launch per size, in clusters of as many CTAs as it has tiles, against the per-order launch, which 16
+    realizations with one of 8 tiles among them take: filtered vectors and moments equal to the last bit, runs of
+    unequal length."""
+    big = {65536: 14, 32768: 13}[tile]
+    sizes = Ns + (big,) * (16 - len(Ns))
+    models = [W.spin_glass_shard(N, seed=190 + r) for r, N in enumerate(sizes)]
+    if flip:
+        models = [_flip(m, 0.5 - 0.07 * r) for r, m in enumerate(models)]
+    psis = [W.start_vectors(N, 4, seed=20, r=r) for r, N in enumerate(sizes)]
+    emax = np.array([_bound(m) for m in models])
+    K, n = 5 + np.arange(16) % 3, 2 + np.arange(16) % 2
+    out = []
+    for count in (len(Ns), 16):
+        d = P.Dacp(models[:count], psis[:count], block_b=4, precision=P.DACP_DF32)
+        try:
+            d.set_launch(0, tile)
+            d.set_params(emax[:count], 0.1 * emax[:count], K[:count], n[:count])
+            d.filter()
+            before = d.launch_count()
+            d.basis_moments()
+            launches = len(set(Ns)) if count == len(Ns) else max(d.params()["kn"]) + 2
+            assert d.launch_count() == before + launches
+            out.append([d.filtered(r) for r in range(len(Ns))] + [d.moments(r) for r in range(len(Ns))])
+        finally:
+            d.close()
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
