@@ -352,14 +352,18 @@ dacp_status dacp_apply_h(dacp_handle hd, int r, const void* x_dev, void* y_dev);
 dacp_status dacp_get_timings(dacp_handle hd, double* ms);
 
 /*
- * dacp_autotune -- pick how the recurrences are launched by timing `orders`
- * evolution orders of this handle's own realizations for every candidate:
+ * dacp_autotune -- pick how the recurrences are launched by timing up to
+ * `orders` orders of this handle's own realizations, with the launches that
+ * dacp_basis_moments would make, for every candidate (dacp_filter's where the
+ * evolution is the fixed-point one of DACP_FP64 handles, which the choice does
+ * not touch):
  * tile size (8 to 128 KB of the vector per CTA) x launch mode (per-order
  * launches replayed from a CUDA graph, one persistent cooperative launch
  * with a grid barrier per order, or -- float32 vectors, where the staged
  * tiles fit shared memory -- graph-replayed launches with staged tiles, mode 2
  * of dacp_set_launch). The fastest is kept and cached for the
- * process, keyed by (sorted N list, b, precision). Needs parameters; resets
+ * process, keyed by (sorted N list, b, precision, pair couplings or none).
+ * Needs parameters; resets
  * filter and moment results (run dacp_filter again). *tile_bytes_out may be
  * NULL.
  */

@@ -859,8 +859,9 @@ dacp_status df_resident_streams(dacp_ctx* c, size_t count) {
 // order[0 .. R), group by group: group g is order[from[g] .. from[g + 1]) (from ends with R) and is done when
 // done[g], a stream, is; done[0] is the handle's. Every size has a launch of its own, with clusters of as many
 // CTAs as it has tiles: 300 filter orders of 512 shards, half of them of 11 and half of 13 spins, take 50.6 ms,
-// 60.7 as per-order launches and 80.8 in clusters of the largest size's. The launches run on streams beside each other, in rising group order and falling size where SMs are short, the
-// longest runs of each first. The streams of groups 1, 2, ... are the first of the handle's extra ones.
+// 60.7 as per-order launches and 80.8 in clusters of the largest size's. The launches run on streams beside each
+// other, in rising group order and falling size where SMs are short, the longest runs of each first. The streams
+// of groups 1, 2, ... are the first of the handle's extra ones.
 dacp_status df_resident_launch(dacp_ctx* c, bool filter, const std::vector<int>& order, const std::vector<int>& from,
                                std::vector<cudaStream_t>* done) {
     TRY(resident_lists(c));
@@ -2587,7 +2588,11 @@ dacp_status dacp_autotune(dacp_handle c, int orders, int* tile_bytes_out) {
     if (orders < 4 || orders > 100000) return fail(c, DACP_ERR_ARG, "orders out of range");
     std::vector<int> ns = c->N;
     std::sort(ns.begin(), ns.end());
-    std::string key = std::to_string(c->b) + "p" + std::to_string(c->prec);
+    // what the choice is for: the evolution, or the filter where the evolution runs in fixed point on its own tiles
+    FxPlan plan;
+    const int maxK = *std::max_element(c->K.begin(), c->K.end());
+    const bool filter = maxK > 0 && fx_usable(c, c->b, &plan);
+    std::string key = std::to_string(c->b) + "p" + std::to_string(c->prec) + (c->has_pairs ? "x" : "") + (filter ? "f" : "");
     for (int v : ns) key += "," + std::to_string(v);
     int best = -1;
     {
@@ -2595,23 +2600,35 @@ dacp_status dacp_autotune(dacp_handle c, int orders, int* tile_bytes_out) {
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) best = it->second;
     }
-    if (best < 0) {
-        const size_t vec_bytes = static_cast<size_t>(c->Dtot) * c->b * c->esz;
+    const int mode0 = c->launch_mode, tile0 = c->tile_bytes;
+    const size_t vec_bytes = static_cast<size_t>(c->Dtot) * c->b * c->esz;
+    int longest = 0;
+    // the launches that a candidate's dacp_filter or dacp_basis_moments makes, cut to `orders` orders
+    auto candidate = [&]() -> dacp_status {
+        const bool resident = !filter && df_resident_usable(c);
+        CK(cudaMemcpyAsync(resident ? c->psiE_d : c->A_d, c->psi0_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
+        CK(cudaEventRecord(c->ev[0], c->st));
+        if (resident) TRY(df_resident_run(c, false));
+        else TRY(run_orders(c, filter, longest));
+        CK(cudaEventRecord(c->ev[1], c->st));
+        CK(cudaStreamSynchronize(c->st));
+        return check_device_flag(c);
+    };
+    auto measure = [&]() -> dacp_status {
+        if (!filter) TRY(set_evolution_coef(c, c->emax));
+        for (RealInfo& R : c->info) {
+            R.nf = std::min(R.nf, orders);
+            R.ne = std::min(R.ne, orders);
+            longest = std::max(longest, filter ? R.nf : R.ne);
+        }
         double best_ms = 1e300;
         for (int cand = 0; cand < 3 * kNumTiles; ++cand) {
             const int tb = kTileCandidates[cand % kNumTiles];
             if (cand / kNumTiles == 2 && !staged_possible(c, tb)) continue;
             c->launch_mode = cand / kNumTiles;
-            TRY(retile(c, tb));
-            TRY(set_evolution_coef(c, c->emax));
-            CK(cudaMemcpyAsync(c->A_d, c->psi0_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
-            TRY(run_orders(c, false, kGraphOrders));         // warm-up; captures the graph
-            CK(cudaMemcpyAsync(c->A_d, c->psi0_d, vec_bytes, cudaMemcpyDeviceToDevice, c->st));
-            CK(cudaEventRecord(c->ev[0], c->st));
-            TRY(run_orders(c, false, orders));
-            CK(cudaEventRecord(c->ev[1], c->st));
-            CK(cudaStreamSynchronize(c->st));
-            TRY(check_device_flag(c));
+            TRY(retile(c, tb));                          // uploads the cut run lengths as well
+            TRY(candidate());                            // warm-up; captures the graph
+            TRY(candidate());
             float ms = 0.f;
             CK(cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]));
             if (ms < best_ms) {
@@ -2619,12 +2636,25 @@ dacp_status dacp_autotune(dacp_handle c, int orders, int* tile_bytes_out) {
                 best = cand;
             }
         }
+        return DACP_OK;
+    };
+    if (best < 0) {
+        const dacp_status s = measure();
+        if (s != DACP_OK) {
+            // the handle as it was: mode, tiles, run lengths and the filter's coefficients
+            const std::string why = c->err;
+            c->launch_mode = mode0;
+            retile(c, tile0);
+            apply_params(c);
+            c->err = why;
+            return s;
+        }
         std::lock_guard<std::mutex> lk(g_tune_mu);
         g_tune_cache[key] = best;
     }
     c->launch_mode = best / kNumTiles;
     TRY(retile(c, kTileCandidates[best % kNumTiles]));
-    TRY(apply_params(c));          // filter coefficients back; results must be recomputed
+    TRY(apply_params(c));          // run lengths and filter coefficients back; results must be recomputed
     if (tile_bytes_out) *tile_bytes_out = kTileCandidates[best % kNumTiles];
     return DACP_OK;
 }

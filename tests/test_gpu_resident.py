@@ -324,3 +324,28 @@ def test_double_float_clusters_of_every_size_keep_the_bits(Ns, tile, flip):
             d.close()
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("N,R", [(13, 8), (11, 36)])
+def test_autotuner_weighs_the_resident_launch(N, R):
+    """A few double-float realizations run twice as fast in clusters as with a launch per order: tuned or not, they
+    take them, and the tuner leaves run lengths and parameters as they were."""
+    models = [W.spin_glass_shard(N, seed=210 + r) for r in range(R)]
+    psis = [W.start_vectors(N, 4, seed=21, r=r) for r in range(R)]
+    emax = np.array([_bound(m) for m in models])
+    d = P.Dacp(models, psis, block_b=4, precision=P.DACP_DF32)
+    try:
+        d.set_params(emax, 0.05 * emax, 7, 6)                 # 378 orders
+        moments = []
+        for tune in (False, True):
+            if tune:
+                d.autotune(64)
+            d.filter()
+            before = d.launch_count()
+            d.basis_moments()
+            assert d.launch_count() == before + 1
+            moments.append([d.moments(r) for r in range(R)])
+        for x, y in zip(*moments):
+            assert x.shape == y.shape and np.abs(x - y).max() <= 8 * (N + 8) * 2.0 ** -44 * 378 ** 2
+    finally:
+        d.close()
