@@ -242,8 +242,10 @@ dacp_status dacp_central_eigs(dacp_handle hd, int n_eigs, double window, double 
  * call, with the subspace solves overlapped with the evolution: realizations
  * finish their evolution at different orders (k_n differs), and each group of
  * finished realizations is solved (batched cuSOLVER / cuBLAS on a second
- * stream, driven by a worker thread) while the rest keep evolving. Results
- * are those of the three separate calls up to the rounding of the batched
+ * stream, driven by a worker thread) while the rest keep evolving. Handles
+ * whose evolution is the fixed-point one hand all realizations over when it
+ * ends: it is short beside the solves, and one batched solve of the whole
+ * batch takes less time than four of its quarters. Results are those of the three separate calls up to the rounding of the batched
  * eigensolver (the batch composition sets the padded size).
  * Arguments and per-realization failures as in dacp_central_eigs. Requires
  * parameters; leaves the handle as dacp_basis_moments does (moments kept for
