@@ -382,9 +382,10 @@ dacp_status dacp_autotune(dacp_handle hd, int orders, int* tile_bytes_out);
  * (DACP_ERR_ARG), as is mode 2 on float64 or double-float vectors. Setting
  * resets filter and moment results. The resident evolution of DACP_FP64
  * handles (see dacp_basis_moments) does not depend on mode and tile size.
- * At the default of 64 KB, DACP_FP64 handles split their vectors further, down
- * to 8 KB, while the batch has fewer tiles than the GPU has SMs, and
- * dacp_apply_h of DACP_FP32 handles uses tiles of 4 to 16 KB.
+ * A new handle has tiles of 64 KB, or of 32 to 8 KB in DACP_FP64 handles of
+ * fewer tiles than the GPU has SMs; dacp_get_launch gives the size in use.
+ * dacp_apply_h of DACP_FP32 handles uses tiles of 4 to 16 KB until
+ * dacp_set_launch sets a size.
  */
 dacp_status dacp_set_launch(dacp_handle hd, int mode, int tile_bytes);
 dacp_status dacp_get_launch(dacp_handle hd, int* mode, int* tile_bytes);

@@ -86,7 +86,8 @@ struct dacp_ctx {
     std::vector<Item> items;
     int64_t Dtot = 0;
     int smem = 0;
-    int tile_bytes = 0;
+    int tile_bytes = 0;                 // of the tiles in use
+    bool tile_set = false;              // as the caller set them (dacp_set_launch)
     int tb_uniform = 0;                 // tile bits shared by every realization, else 0
     std::vector<double> J_h, h_h, g_h;   // [R][kMaxSpins(^2)]
     std::vector<double> pnorm;          // Pauli 1-norm of each H: clamp of the E_max bound
@@ -478,9 +479,8 @@ dacp_status run_orders(dacp_ctx* c, bool filter, int orders,
 // 12-spin chain 646 and 119 ms; one product with H, call included, 37 and 26 us at 10 spins, 65 and 33 at 16,
 // 70 and 65 at 18. Past one tile per SM the gain is small (20 spins: 207 at 64 KB, 188 at 32 KB) and the
 // moments pay per tile.
-void tile_geometry(dacp_ctx* c, int tile_bytes) {
-    c->tile_bytes = tile_bytes;
-    if (c->prec == kPrecF64 && tile_bytes == kTileBytes) {
+void tile_geometry(dacp_ctx* c, int tile_bytes, bool by_default) {
+    if (c->prec == kPrecF64 && by_default) {
         auto tiles = [&](int bytes) {
             int64_t n = 0;
             for (int r = 0; r < c->R; ++r)
@@ -489,6 +489,7 @@ void tile_geometry(dacp_ctx* c, int tile_bytes) {
         };
         while (tile_bytes > kMinTileBytes && tiles(tile_bytes) < 152) tile_bytes /= 2;
     }
+    c->tile_bytes = tile_bytes;
     int tb_cap = 0;
     while ((static_cast<int64_t>(2) << tb_cap) * c->b * static_cast<int64_t>(c->esz) <= tile_bytes) ++tb_cap;
     c->items.clear();
@@ -512,8 +513,8 @@ size_t part_slots(const dacp_ctx* c) { return c->items.size() * 2 * c->b * c->b 
 
 // Float32 tiles of dacp_apply_h, which reads the vector once and keeps nothing: 1/128 of the vector, at least
 // 4 KB, at most 16 KB, against 64 KB for the recurrences, whose moments pay per tile. 16 KB and 64 KB tiles take
-// 26 and 37 us on 2^16 states at b = 4, 31 and 44 us on 2^18, 48 and 51 us on 2^20, call included. A tile
-// size that the caller set is kept.
+// 26 and 37 us on 2^16 states at b = 4, 31 and 44 us on 2^18, 48 and 51 us on 2^20, call included.
+// dacp_set_launch takes its own tile size here too.
 dacp_status apply_geometry(dacp_ctx* c) {
     std::vector<Item> items;
     c->apply_info = c->info;
@@ -546,7 +547,7 @@ dacp_status apply_geometry(dacp_ctx* c) {
 // as they were.
 dacp_status retile(dacp_ctx* c, int tile_bytes) {
     const int before = c->tile_bytes;
-    tile_geometry(c, tile_bytes);
+    tile_geometry(c, tile_bytes, false);
     Item* items = nullptr;
     double* part = nullptr;
     const size_t slots = part_slots(c);
@@ -563,7 +564,7 @@ dacp_status retile(dacp_ctx* c, int tile_bytes) {
     if (s != DACP_OK) {
         dfree(c, items);
         dfree(c, part);
-        tile_geometry(c, before);
+        tile_geometry(c, before, false);
         return s;
     }
     dfree(c, c->items_d);
@@ -1079,7 +1080,7 @@ dacp_status dacp_create(dacp_handle* out, int n_real, const int* n_spins, const 
     }
     c->Dtot = off;
     c->pnorm0 = c->pnorm;
-    tile_geometry(c, kTileBytes);
+    tile_geometry(c, kTileBytes, true);
     c->emax.assign(n_real, 0.0);
     c->a.assign(n_real, 0.0);
     c->K.assign(n_real, 0);
@@ -2550,7 +2551,7 @@ dacp_status dacp_apply_h(dacp_handle c, int r, const void* x_dev, void* y_dev) {
     a.out = static_cast<char*>(y_dev) - shift;
     const RealInfo* info = &c->info[r];
     int smem = c->smem;
-    if (c->fp32 && c->tile_bytes == kTileBytes) {
+    if (c->fp32 && !c->tile_set) {
         info = &c->apply_info[r];
         smem = c->apply_smem;
         a.items = c->apply_items_d;
@@ -2658,6 +2659,7 @@ dacp_status dacp_autotune(dacp_handle c, int orders, int* tile_bytes_out) {
     c->launch_mode = best / kNumTiles;
     TRY(retile(c, kTileCandidates[best % kNumTiles]));
     TRY(apply_params(c));          // run lengths and filter coefficients back; results must be recomputed
+    c->tile_set = false;
     if (tile_bytes_out) *tile_bytes_out = kTileCandidates[best % kNumTiles];
     return DACP_OK;
 }
@@ -2672,6 +2674,7 @@ dacp_status dacp_set_launch(dacp_handle c, int mode, int tile_bytes) {
         return fail(c, DACP_ERR_ARG, "staged tiles of %d bytes exceed shared memory", tile_bytes);
     c->launch_mode = mode;
     TRY(retile(c, tile_bytes));
+    c->tile_set = true;
     if (c->state > 1) c->state = 1;
     return DACP_OK;
 }

@@ -349,3 +349,26 @@ def test_autotuner_weighs_the_resident_launch(N, R):
             assert x.shape == y.shape and np.abs(x - y).max() <= 8 * (N + 8) * 2.0 ** -44 * 378 ** 2
     finally:
         d.close()
+
+
+@pytest.mark.parametrize("b,N", [(4, 10), (1, 13), (4, 13)])
+def test_a_tile_size_that_the_caller_sets_is_the_one_in_use(N, b):
+    """Small float64 handles start with smaller tiles than 64 KB, and say so; 64 KB are 64 KB when asked for.
+    The filtered vectors do not depend on the tiles, but for the sum of their norm."""
+    m = W.chain(N)
+    psi = W.start_vectors(N, b, seed=22)
+    d = P.Dacp([m], [psi], block_b=b, precision=P.DACP_FP64)
+    try:
+        first = d.launch()
+        assert first == (0, 8192)
+        emax = np.array([_bound(m)])
+        d.set_params(emax, 0.2 * emax, 6, 2)
+        ref = None
+        for tile in (first[1], 65536, 16384, 65536):
+            d.set_launch(0, tile)
+            assert d.launch() == (0, tile)
+            d.filter()
+            ref = d.filtered(0) if ref is None else ref
+            assert np.abs(d.filtered(0) - ref).max() <= 1e-14       # normalised; the norm's sum is regrouped
+    finally:
+        d.close()
