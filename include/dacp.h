@@ -598,7 +598,7 @@ dacp_status dacp_get_features(dacp_handle hd, float* feats, int64_t cap);
  * them).
  *
  *   n_spins      N, 1 <= N <= 16; larger N returns DACP_ERR_ARG (the scratch
- *                array below holds 4 x 2^16 float64 states).
+ *                array below holds 3 x 2^16 float64 states).
  *   J, h, gamma  host arrays as in dacp_create for one realization (J is
  *                N x N row-major, only i<j read).
  *   emax         bound on |E|; G = H / emax.
@@ -608,20 +608,22 @@ dacp_status dacp_get_features(dacp_handle hd, float* feats, int64_t cap);
  *   mu_dev       device pointer, 2 * n_orders float64: on return
  *                mu_j = <psi| T_j(G) |psi>, j = 0 .. 2 n_orders - 1, from the
  *                same evolution as dacp_basis_moments of a DACP_FP64 handle.
- *                It may overlap psi_dev.
+ *                It may overlap psi_dev, which is then kept in host memory
+ *                during the call.
  *   stream       cudaStream_t or NULL. The call copies J, h, gamma and its
  *                run lengths from host memory into the scratch array on this
  *                stream, and waits for the stream before it returns.
  *
- * Scratch: one file-scope device array of about 2.1 MB (vectors, diagonal,
+ * Scratch: one file-scope device array of about 1.6 MB (vectors, diagonal,
  * couplings, partial sums, counters), held by every GPU that loads the
  * library until the process exits. The first call on a device does the
  * set-up: it looks up the array's address (cudaGetSymbolAddress) and raises
- * the stencil kernel's shared-memory limit; make that first call before any
- * stream capture. Every call overwrites the array and clears its counters,
- * and two calls that overlap on the GPU (different streams or threads) race
+ * the shared-memory limits of the kernels, which are the same for every size;
+ * make that first call before any stream capture. Every call overwrites the
+ * array and clears its counters, and two calls that overlap on the GPU (different streams or threads) race
  * on it and corrupt each other's results: serialise them.
- * Returns DACP_OK, DACP_ERR_ARG, DACP_ERR_CUDA or DACP_ERR_TIMEOUT.
+ * Returns DACP_OK, DACP_ERR_ARG, DACP_ERR_CUDA, DACP_ERR_TIMEOUT or, when the
+ * buffers overlap, DACP_ERR_NOMEM (host memory).
  */
 dacp_status dacp_moments_noalloc(int n_spins, const double* J, const double* h, const double* gamma,
                                  double emax, const double* psi_dev, int n_orders, double* mu_dev,

@@ -20,7 +20,9 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <memory>
 #include <mutex>
+#include <new>
 
 #include "../../include/dacp.h"
 #include "common.cuh"
@@ -48,8 +50,7 @@ constexpr int64_t kRegItems = kRegInfo + 32;              // Item[kNaMaxItems]
 constexpr int64_t kRegCount = kRegItems + kNaMaxItems + 32;     // counters (unsigned / int)
 constexpr int64_t kRegEmax = kRegCount + 32;              // E_max
 constexpr int64_t kRegPro = kRegEmax + 32;                // scale exchange of the resident evolution
-constexpr int64_t kRegPsi = kRegPro + (2 << kFxMaxLg);    // start vector, when the moments are written over it
-constexpr int64_t kNaTotal = kRegPsi + kNaStates;
+constexpr int64_t kNaTotal = kRegPro + (2 << kFxMaxLg);
 
 static_assert(sizeof(RealInfo) <= 32 * sizeof(double), "RealInfo region too small");
 static_assert(sizeof(Item) * kNaMaxItems <= (kNaMaxItems + 32) * sizeof(double), "Item region too small");
@@ -84,7 +85,8 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 128) return DACP_ERR_CUDA;
 
     // Set-up, once per device, with that device current: the scratch address
-    // and the shared-memory attribute of the stencil kernel.
+    // and the shared-memory attribute of the stencil kernel (that of the
+    // resident one, the same for every size, comes with its first launch).
     double* base = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_na_mu);
@@ -141,14 +143,22 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
     const RealInfo* info_d = reinterpret_cast<const RealInfo*>(base + kRegInfo);
     if (launch_diag(kPrecF64, info_d, 0, N, base + kRegJ, base + kRegH, base + kRegDiag, st) != cudaSuccess)
         return DACP_ERR_CUDA;
-    // callers that count every byte may hand in overlapping buffers: the start vector is read after moments are written
+    // Callers that count every byte may hand in overlapping buffers. The first run reads the start vector before it
+    // writes a moment; for a second one the vector is kept on the host.
+    const size_t psi_bytes = sizeof(double) * static_cast<size_t>(D);
     const uintptr_t psi_at = reinterpret_cast<uintptr_t>(psi_dev), mu_at = reinterpret_cast<uintptr_t>(mu_dev);
-    const double* psi = psi_dev;
-    if (psi_at < mu_at + 2 * sizeof(double) * n_orders && mu_at < psi_at + sizeof(double) * D) {
-        if (!ok(cudaMemcpyAsync(base + kRegPsi, psi_dev, sizeof(double) * D, cudaMemcpyDeviceToDevice, st)))
+    std::unique_ptr<double[]> kept;
+    if (psi_at < mu_at + 2 * sizeof(double) * n_orders && mu_at < psi_at + psi_bytes) {
+        kept.reset(new (std::nothrow) double[D]);
+        if (!kept) return DACP_ERR_NOMEM;
+        if (!ok(cudaMemcpyAsync(kept.get(), psi_dev, psi_bytes, cudaMemcpyDeviceToHost, st)) ||
+            !ok(cudaStreamSynchronize(st)))
             return DACP_ERR_CUDA;
-        psi = base + kRegPsi;
     }
+    auto psi_to_scratch = [&]() {
+        return kept ? ok(cudaMemcpyAsync(base + kRegA, kept.get(), psi_bytes, cudaMemcpyHostToDevice, st))
+                    : ok(cudaMemcpyAsync(base + kRegA, psi_dev, psi_bytes, cudaMemcpyDeviceToDevice, st));
+    };
 
     // the resident fixed-point evolution, again at its coarse scale if the vectors outgrow the first; what neither
     // suits runs in floating point
@@ -161,7 +171,7 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
         f.real = info_d;
         f.diag = base + kRegDiag;
         f.gam = base + kRegGam;
-        f.psi = psi;
+        f.psi = psi_dev;
         f.emax = base + kRegEmax;
         f.pub0 = reinterpret_cast<int4*>(base + kRegA);
         f.pub1 = reinterpret_cast<int4*>(base + kRegB);
@@ -173,6 +183,10 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
         f.err_flag = reinterpret_cast<int*>(counters + 3);
         for (f.coarse = 0; f.coarse < 2; ++f.coarse) {
             if (f.coarse && !ok(cudaMemsetAsync(counters + 3, 0, 5 * sizeof(unsigned), st))) return DACP_ERR_CUDA;
+            if (f.coarse && kept) {              // every thread reads a slot of w_0 before it publishes it there
+                if (!psi_to_scratch()) return DACP_ERR_CUDA;
+                f.psi = base + kRegA;
+            }
             if (launch_evolve_fx(1, plan, f, 1, st) != cudaSuccess) return DACP_ERR_CUDA;
             noalloc_moments_from_products<<<(n + 255) / 256, 256, 0, st>>>(mu_dev, n);
             unsigned words[5];                   // error flag .. status
@@ -185,9 +199,7 @@ extern "C" dacp_status dacp_moments_noalloc(int n_spins, const double* J, const 
             if (words[4] == kFxUnsuited) break;
         }
     }
-    if (!ok(cudaMemsetAsync(counters + 4, 0, sizeof(unsigned), st)) ||
-        !ok(cudaMemcpyAsync(base + kRegA, psi, sizeof(double) * D, cudaMemcpyDeviceToDevice, st)))
-        return DACP_ERR_CUDA;
+    if (!ok(cudaMemsetAsync(counters + 4, 0, sizeof(unsigned), st)) || !psi_to_scratch()) return DACP_ERR_CUDA;
     StepArgs a;
     memset(&a, 0, sizeof(a));
     a.items = reinterpret_cast<const Item*>(base + kRegItems);
