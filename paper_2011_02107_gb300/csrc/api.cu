@@ -81,6 +81,7 @@ struct dacp_ctx {
     cudaStream_t st = nullptr;
     bool own_stream = false;
     int device = 0;
+    int sms = 0;
     std::vector<int> N;
     std::vector<RealInfo> info;
     std::vector<Item> items;
@@ -487,7 +488,7 @@ void tile_geometry(dacp_ctx* c, int tile_bytes, bool by_default) {
                 n += std::max<int64_t>(1, ((static_cast<int64_t>(c->b) * 8) << c->info[r].N) / bytes);
             return n;
         };
-        while (tile_bytes > kMinTileBytes && tiles(tile_bytes) < 152) tile_bytes /= 2;
+        while (tile_bytes > kMinTileBytes && tiles(tile_bytes) < c->sms) tile_bytes /= 2;
     }
     c->tile_bytes = tile_bytes;
     int tb_cap = 0;
@@ -584,14 +585,15 @@ dacp_status retile(dacp_ctx* c, int tile_bytes) {
     return DACP_OK;
 }
 
-// A stencil CTA whose bounded wait on its tile copy gave up sets err_d.
+// A CTA whose bounded wait gave up sets err_d: 1 for a tile copy, 2 for a barrier.
 dacp_status check_device_flag(dacp_ctx* c) {
     int e = 0;
     CK(cudaMemcpyAsync(&e, c->err_d, sizeof(int), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
     if (e) {
         CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
-        return fail(c, DACP_ERR_TIMEOUT, "a tile copy did not complete within the wait limit");
+        return fail(c, DACP_ERR_TIMEOUT, "%s within the wait limit",
+                    e == 2 ? "a barrier between the CTAs of a launch did not open" : "a tile copy did not complete");
     }
     return DACP_OK;
 }
@@ -816,13 +818,13 @@ dacp_status fx_evolve(dacp_ctx* c, const FxPlan& plan, const FxRun& q, const std
 
 // Whether the recurrences of launch mode 0 run as resident double-float clusters, one CTA per tile of the
 // per-order launch (whose bits they keep). Clusters of up to 4 CTAs win at every batch size: 4.11 against
-// 8.00 ms for 361 evolution orders of 36 13-spin sectors, 61.4 against 64.8 ms of 512. Of 8 CTAs only 15 fit
-// the GPU (120 of 152 SMs), so there the per-order launch is ahead once they do not all run at once: 79.1
-// against 65.2 ms for 256 14-spin shards.
+// 8.00 ms for 361 evolution orders of 36 13-spin sectors, 61.4 against 64.8 ms of 512. Of 8 CTAs few fit the GPU
+// at once (120 of its 152 SMs), so there the per-order launch is ahead once they do not: 79.1 against 65.2 ms for
+// 256 14-spin shards.
 bool df_resident_usable(const dacp_ctx* c) {
     if (c->prec != kPrecDF32 || c->b != 4 || c->has_pairs || c->launch_mode != 0) return false;
     const int max_N = *std::max_element(c->N.begin(), c->N.end());
-    return df4_resident_fits(c->tb_uniform, max_N) && (max_N - c->tb_uniform < 3 || c->R <= 15);
+    return df4_resident_fits(c->tb_uniform, max_N) && (max_N - c->tb_uniform < 3 || c->R <= df4_resident_clusters(c->tb_uniform, 3));
 }
 
 DfResArgs df_resident_args(const dacp_ctx* c) {
@@ -1028,6 +1030,7 @@ dacp_status dacp_create(dacp_handle* out, int n_real, const int* n_spins, const 
         return s;
     };
     cudaGetDevice(&c->device);
+    cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
     c->R = n_real;
     c->b = block_b;
     c->prec = precision == DACP_FP32 ? kPrecF32 : (precision == DACP_DF32 ? kPrecDF32 : kPrecF64);

@@ -80,6 +80,7 @@ struct DfResArgs {
 };
 constexpr int kDfPartSums = 4 * 32; // doubles of DfResArgs::part per CTA
 bool df4_resident_fits(int tbits_uniform, int max_N);
+int df4_resident_clusters(int tbits, int lg);
 cudaError_t launch_df4_resident(int tbits, bool filter, const DfResArgs& a, int count, cudaStream_t st);
 bool df1_resident_fits(int tbits_uniform, int max_N);
 cudaError_t launch_moments_df1_resident(int tbits, const DfResArgs& a, int count, int max_N, int orders, int rows_fixed,

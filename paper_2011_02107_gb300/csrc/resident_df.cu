@@ -485,24 +485,44 @@ cudaError_t launch_moments_df1(const DfResArgs& a, int count, int max_N, int ord
     return cudaGetLastError();
 }
 
+// Launch shape of `count` clusters of 2^lg CTAs; at: room for the cluster attribute.
+cudaLaunchConfig_t df4_config(int TB, bool filter, int count, int lg, cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(count) << lg);
+    cfg.blockDim = dim3(kDfThreads);
+    cfg.dynamicSmemBytes = (filter ? 104 : 72) << TB;     // three or two vectors of 32 bytes a state, and the diagonal
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1u << lg;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = lg > 0 ? 1 : 0;
+    return cfg;
+}
+
 template <int TB>
 cudaError_t launch_df4_resident(bool filter, const DfResArgs& a, int count, cudaStream_t st) {
     auto* f = filter ? filter_df4_resident_kernel<TB> : evolve_df4_resident_kernel<TB>;
-    const int smem = (filter ? 104 : 72) << TB;     // three or two vectors of 32 bytes a state, and the diagonal
-    cudaError_t e = grow_smem_attr(reinterpret_cast<const void*>(f), smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(count) << a.lg);
-    cfg.blockDim = dim3(kDfThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1u << a.lg;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = a.lg > 0 ? 1 : 0;
+    cudaLaunchConfig_t cfg = df4_config(TB, filter, count, a.lg, at);
+    cfg.stream = st;
+    cudaError_t e = grow_smem_attr(reinterpret_cast<const void*>(f), static_cast<int>(cfg.dynamicSmemBytes));
+    if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, f, a);
+}
+
+// Clusters of 2^lg CTAs of the filter, which takes the more shared memory, that the device holds at once.
+template <int TB>
+int df4_clusters(int lg) {
+    auto* f = filter_df4_resident_kernel<TB>;
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = df4_config(TB, true, 1, lg, at);
+    int n = 0;
+    if (grow_smem_attr(reinterpret_cast<const void*>(f), static_cast<int>(cfg.dynamicSmemBytes)) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
 }
 
 }  // namespace
@@ -511,6 +531,14 @@ cudaError_t launch_df4_resident(bool filter, const DfResArgs& a, int count, cuda
 // memory: 147 KB, with the filter's third vector 213 KB), at most 8 of them to a realization (a portable cluster).
 bool df4_resident_fits(int tbits_uniform, int max_N) {
     return (tbits_uniform == 10 || tbits_uniform == 11) && max_N - tbits_uniform <= 3;
+}
+
+int df4_resident_clusters(int tbits, int lg) {
+    switch (tbits) {
+        case 10: return df4_clusters<10>(lg);
+        case 11: return df4_clusters<11>(lg);
+    }
+    return 0;
 }
 
 // Filter or evolve the realizations a.list[0 .. count) in 2^a.lg CTAs each.

@@ -372,3 +372,17 @@ def test_a_tile_size_that_the_caller_sets_is_the_one_in_use(N, b):
             assert np.abs(d.filtered(0) - ref).max() <= 1e-14       # normalised; the norm's sum is regrouped
     finally:
         d.close()
+
+
+def test_a_barrier_that_ran_out_is_named():
+    m = W.spin_glass_shard(9, seed=1)
+    d = P.Dacp([m], [W.start_vectors(9, 1, seed=2)], block_b=1, precision=P.DACP_FP32)
+    try:
+        d.set_params(_bound(m), 0.2 * _bound(m), 4, 2)
+        d.set_launch(1, 2048)
+        P.dacp_test_poison_barrier(d.handle)
+        with pytest.raises(P.DacpError, match="barrier") as e:
+            d.filter()
+        assert e.value.status == 5
+    finally:
+        d.close()
