@@ -258,6 +258,8 @@ dacp_status ensure_batch(dacp_mlp_ctx* c, int B) {
     cudaFree(c->tb);
     cudaFree(c->yb);
     c->act.assign(c->sizes.size(), nullptr);
+    c->delta = c->xb = c->tb = c->yb = nullptr;      // an allocation below may fail: nothing freed stays in use
+    c->cap_b = 0;
     int64_t W = 0;
     for (size_t l = 1; l < c->sizes.size(); ++l) W += c->sizes[l];
     for (size_t l = 0; l < c->sizes.size(); ++l) MCK(cudaMalloc(&c->act[l], sizeof(float) * B * c->sizes[l]));
