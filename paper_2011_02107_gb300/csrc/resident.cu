@@ -155,7 +155,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     __shared__ FxSum red_s[kFxRedRing][kFxThreads / 32][NS];
     __shared__ float pro_s[3][kFxThreads / 32];
     __shared__ float max_s[4];
-    __shared__ int stop_s;                         // the group's status, read once in kFxCheck orders
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nwork = blockDim.x, nwarps = nwork >> 5;
@@ -321,7 +320,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
     // while order k's barrier is open: the CTA's sums of order k - 1, and the rows of order k - 3, whose
     // partials every CTA wrote before barrier k - 1. The warp may run behind by one order, hence the rings.
     auto moments_behind = [&](const int k) {
-        if (lane == 31 && k % kFxCheck == 2) stop_s = __ldcg(a.status + group);    // as of order k - 3
         if (active && lane < NS && k >= 1 && k <= orders) {
             long long hi = 0, lo = 0;
             for (int w = 0; w < nwarps; ++w) {
@@ -514,10 +512,11 @@ __global__ void __launch_bounds__(kFxThreads, 1) evolve_fx_kernel(const FxArgs a
         const int k1 = k0 + kFxCheck < orders ? k0 + kFxCheck : orders;
         for (int k = k0; k < k1; ++k)
             if (!order(k)) return;
-        if (chk) a.status[group] = kFxOutgrown;
-        // the flag as it stood before this stretch (moments_behind), the same at every CTA of the group: the stretch's
-        // own is seen in the next one. (A look at every order takes 0.1 to 0.5 us of its 2 to 3.)
-        if (k0 > 0 && stop_s) return;
+        // Outgrown in an earlier stretch? (The status is the larger the earlier: this stretch's, which some CTAs may
+        // have set already, does not count, so that all CTAs of the group leave together.) A look at every order
+        // would take 0.1 to 0.5 us of its 2 to 3.
+        if (__ldcg(a.status + group) > 0x7fffffff - k0) return;
+        if (chk) atomicMax(a.status + group, 0x7fffffff - k0);
     }
     for (int k = orders; k < orders + 3; ++k)
         if (!fx_group_sync(a, group, target += G, [&] { moments_behind(k); })) return;
