@@ -110,6 +110,8 @@ DF32_TRAFFIC_SOURCE = "stored ncu capture of the current kernel, one launch, not
 # two float32 lane operations each.
 DF_FMA_OPS, DF_SUB_OPS = 12, 8
 FP32_LANES_PER_SM = 128
+WIDE_IMADS_PER_SM = 30     # 32 x 32 -> 64-bit integer multiply-adds per clock and SM, dependent operands, measured
+FX_MAX_VALUES = 1 << 20    # largest realization of the resident float64 evolution
 
 
 def sm_count():
@@ -128,9 +130,11 @@ def roofline(wl, n_real, phase, bytes_evo, states_evo, clk, sms, launch_mode=0, 
     symmetric) double-float multiply-adds x DF_FMA_OPS float32 lane operations,
     plus b subtractions of w_{k-1} x DF_SUB_OPS, against the device's SMs x 128
     lanes x the SM clock sampled during the run.
-    float64: the same multiply-add count against the measured float64 dgemm
-    rate (1.10 TFLOP/s = 0.55 T FMA/s on this GB300); the evolution runs in fixed
-    point on the integer pipe, so the fraction may exceed 1.
+    float64, resident (up to 2^20 values a realization): integer-pipe bound; a
+    product of two fixed-point values is three wide multiply-adds, the
+    subtraction of w_{k-1} two, against 30 of them per clock and SM (measured).
+    float64, larger: FP64-pipe bound; the same multiply-add count against the
+    measured float64 dgemm rate (1.10 TFLOP/s = 0.55 T FMA/s on this GB300).
     sectors: the recurrences run on the parity sectors, N - 1 spins whose
     N - 1 x-fields and one global flip make N flip terms per state.
     """
@@ -147,7 +151,7 @@ def roofline(wl, n_real, phase, bytes_evo, states_evo, clk, sms, launch_mode=0, 
     df_ops_per_state = DF_FMA_OPS * (N * b + b + b * (b + 1)) + DF_SUB_OPS * b
     kern = {"fp32": "step_kernel<float,4,kEvolve>",
             "df32": "step_kernel_df4tb<kEvolve,11> (double-float, b = 4, paired float32 instructions)",
-            "fp64": f"evolve_fx_kernel<{b}> (59-bit fixed point on the integer pipe, vectors in shared memory)"}[wl["prec"]]
+            "fp64": f"step_kernel<double,{b},kEvolve>"}[wl["prec"]]
     if wl["prec"] == "df32" and sectors and launch_mode == 0:
         kern = "evolve_df4_resident_kernel<11> (double-float, b = 4, a cluster per sector, vectors in shared memory)"
     if wl["prec"] == "fp32":
@@ -174,6 +178,18 @@ def roofline(wl, n_real, phase, bytes_evo, states_evo, clk, sms, launch_mode=0, 
                 "peak_source": f"{sms} SMs x 128 float32 lanes x {mhz:.0f} MHz (sampled)",
                 "algorithmic": f"{DF_FMA_OPS} x {N * b + b + b * (b + 1)} double-float FMA + {DF_SUB_OPS} x {b} "
                                f"subtractions = {df_ops_per_state} float32 lane operations per state and order"}
+    if b << N <= FX_MAX_VALUES:
+        kern = f"evolve_fx_kernel<{b}> (59-bit fixed point on the integer pipe, vectors in shared memory)"
+        imads_per_state = 3 * (N * b + b + b * (b + 1)) + 2 * b
+        mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz") or 2070.0
+        peak = sms * WIDE_IMADS_PER_SM * mhz * 1e6 / 1e12            # T wide multiply-adds/s
+        achieved = states_evo * imads_per_state / t_e / 1e12 if t_e > 0 else None
+        return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "T wide integer multiply-adds/s",
+                "frac": achieved / peak if achieved else None, "traffic": None, "kernel": kern,
+                "peak_source": f"{sms} SMs x {WIDE_IMADS_PER_SM} 32 x 32 -> 64-bit multiply-adds per clock (measured) "
+                               f"x {mhz:.0f} MHz (sampled)",
+                "algorithmic": f"3 x {N * b + b + b * (b + 1)} products + 2 x {b} subtractions = {imads_per_state} wide "
+                               "integer multiply-adds per state and order"}
     peak = 0.55                                                         # T FMA/s, measured dgemm
     achieved = states_evo * fma_per_state / t_e / 1e12 if t_e > 0 else None
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "T float64 FMA/s",

@@ -53,6 +53,21 @@ def test_roofline_arithmetic():
     assert r["bound"] == "hbm" and abs(r["achieved"] - 3000.0) < 1e-9 and r["unit"] == "GB/s"
 
 
+def test_roofline_of_the_fixed_point_evolution():
+    """Integer work against the integer pipe: three wide multiply-adds a product, two for w_(k-1); realizations
+    beyond the resident form against the float64 pipe."""
+    sys.path.insert(0, ROOT)
+    import bench as B
+    wl = dict(B.WORKLOADS["c2"], prec="fp64")
+    N, b = wl["N"], wl["b"]
+    r = B.roofline(wl, 1, [0.0, 1000.0, 0.0], 3e12, 1e9, {"sm_mhz": 2000.0}, 152)
+    assert (b << N) <= 1 << 20 and r["kernel"].startswith("evolve_fx_kernel")
+    assert abs(r["achieved"] - 1e-3 * (3 * (N * b + b + b * (b + 1)) + 2 * b)) < 1e-12
+    assert abs(r["peak"] - 152 * 30 * 2000e6 / 1e12) < 1e-9 and abs(r["frac"] - r["achieved"] / r["peak"]) < 1e-12
+    r = B.roofline(dict(wl, N=21), 1, [0.0, 1000.0, 0.0], 3e12, 1e9, {"sm_mhz": 2000.0}, 152)
+    assert r["kernel"].startswith("step_kernel<double") and r["peak"] == 0.55
+
+
 def test_sector_levels_rule():
     """Each parity sector is asked for half of n_eigs plus a margin of 1 % (at least 5 levels);
     --sector-share overrides it."""
