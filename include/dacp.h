@@ -180,7 +180,9 @@ dacp_status dacp_set_params(dacp_handle hd, const double* emax, const double* a,
  *   K:     ceil(c_order * E_max / a) (Sec. II A: c_order = 18). c_order <= 0
  *          picks the precision default: 18 for DACP_FP64 and DACP_DF32, 6 for DACP_FP32
  *          (float32 moments resolve a dynamic range of about e^12).
- * Errors: DACP_ERR_ARG, DACP_ERR_CUDA.
+ * Its device scratch (and that of the dacp_get_* read-backs) stays with the
+ * handle up to 64 MB; larger scratch is allocated for the call.
+ * Errors: DACP_ERR_ARG, DACP_ERR_CUDA, DACP_ERR_NOMEM.
  */
 dacp_status dacp_choose_params(dacp_handle hd, int n_eigs, double d_ratio,
                                double basis_ratio, double c_order,
