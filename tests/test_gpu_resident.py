@@ -386,3 +386,25 @@ def test_a_barrier_that_ran_out_is_named():
         assert e.value.status == 5
     finally:
         d.close()
+
+
+@pytest.mark.parametrize("b", [1, 2, 4])
+@pytest.mark.parametrize("bits,N", [(9, 9), (9, 12), (10, 11), (10, 13), (11, 13)])
+def test_kpm_moments_keep_the_bits_at_every_tile_size(bits, N, b):
+    """As above for tiles of 2^9 to 2^11 states, one to eight of them, and every block size."""
+    models = [_flip(W.spin_glass_shard(n, seed=220 + n), 0.3) for n in (N, 14)]
+    psis = [W.start_vectors(m["N"], b, seed=23, r=r) for r, m in enumerate(models)]
+    out = []
+    for count in (1, 2):
+        d = P.Dacp(models[:count], psis[:count], block_b=b, precision=P.DACP_DF32)
+        try:
+            d.set_launch(0, (8 * b) << bits)
+            before = d.launch_count()
+            d.choose_params(12)
+            p = d.params()
+            out.append([d.launch_count() - before, np.asarray(p["a"])[0], np.asarray(p["emax"])[0],
+                        np.asarray(d.features())[0]])
+        finally:
+            d.close()
+    assert out[1][0] == out[0][0] + 127                   # 128 per-order launches in the place of one
+    assert all(np.array_equal(x, y) for x, y in zip(out[0][1:], out[1][1:]))
